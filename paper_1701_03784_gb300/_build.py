@@ -9,7 +9,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpic_gb300.so")
 SOURCES = ["mesh.cpp", "spai.cpp", "sources.cpp", "sim.cu", "k_push.cu", "k_push_f32.cu", "k_field.cu",
-           "k_sort.cu", "k_diag.cu", "k_emit.cu", "k_probe.cu", "mlp.cu", "k_mlp_tc.cu"]
+           "k_sort.cu", "k_diag.cu", "k_emit.cu", "k_probe.cu", "mlp.cu", "k_mlp_f32.cu",
+           "k_mlp_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "nvcc")
 
@@ -25,7 +26,8 @@ def _flags(src):
 def _compile(src, verbose=False):
     obj = os.path.join(BUILD, src + ".o")
     path = os.path.join(CSRC, src)
-    deps = [path, os.path.join(CSRC, "pic_internal.h"), os.path.join(HERE, "..", "include", "pic.h")]
+    deps = [path, os.path.join(HERE, "..", "include", "pic.h")]
+    deps += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
     if os.path.exists(obj) and os.path.getmtime(obj) >= max(os.path.getmtime(d) for d in deps):
         return obj
     cmd = [NVCC] + _flags(src) + ["-c", path, "-o", obj]

@@ -1,11 +1,13 @@
 // Surrogate network ensemble: small multilayer perceptrons (tanh-GELU hidden layers, linear
 // output) that map sweep parameters to simulation outputs, trained and evaluated on the
-// GPU by the kernels in this file (FP32 on CUDA cores) and k_mlp_tc.cu (BF16 tensor-core
+// GPU by the kernels in k_mlp_f32.cu (FP32 on CUDA cores) and k_mlp_tc.cu (BF16 tensor-core
 // inference, and optionally the training products: pic_mlp_set_training).  The paper has
 // no counterpart.
 //
 // Layout: per member, the layers' parameters one after another, W_l (n_out x n_in,
-// row-major) then b_l; members follow each other at a fixed stride.  Activations are
+// row-major) then b_l, each starting on a 16-byte boundary (the copies into shared memory
+// are 16 bytes wide); members follow each other at a fixed stride.  The caller's arrays
+// are without the padding.  Activations are
 // row-major (sample x unit) per member.  Minibatch indices come from a counter-based hash
 // of (seed, member, step, row), so a training run is reproducible.
 #include <algorithm>
@@ -13,14 +15,12 @@
 #include <cstring>
 #include <vector>
 
+#include "mlp_math.h"
 #include "pic_internal.h"
 
 namespace pic {
 
 namespace {
-constexpr int GT = 16;           // GEMM tile
-constexpr float C_GELU = 0.7978845608028654f;   // sqrt(2/pi)
-
 // C(z)[m][n] (+)= sum_k A(z, m, k) B(z, k, n), operands addressed by strides; z = member
 struct GemmArgs {
     const float *A, *B;
@@ -30,38 +30,6 @@ struct GemmArgs {
     int sAm, sAk, sBk, sBn, ldc;
     int accumulate;
 };
-
-__global__ void __launch_bounds__(GT * GT) k_gemm(GemmArgs g) {
-    __shared__ float As[GT][GT + 1], Bs[GT][GT + 1];
-    const int z = blockIdx.z;
-    const float *A = g.A + z * g.sAz, *B = g.B + z * g.sBz;
-    float *C = g.C + z * g.sCz;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int m = blockIdx.y * GT + ty, n = blockIdx.x * GT + tx;
-    float acc = 0.f;
-    for (int k0 = 0; k0 < g.K; k0 += GT) {
-        const int ka = k0 + tx, kb = k0 + ty;
-        const int ma = blockIdx.y * GT + ty;
-        As[ty][tx] = (ma < g.M && ka < g.K) ? A[(long long)ma * g.sAm + (long long)ka * g.sAk] : 0.f;
-        Bs[ty][tx] = (kb < g.K && n < g.N) ? B[(long long)kb * g.sBk + (long long)n * g.sBn] : 0.f;
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GT; kk++) acc = fmaf(As[ty][kk], Bs[kk][tx], acc);
-        __syncthreads();
-    }
-    if (m < g.M && n < g.N) {
-        float *c = C + (long long)m * g.ldc + n;
-        *c = g.accumulate ? *c + acc : acc;
-    }
-}
-
-__device__ __forceinline__ float gelu(float z) {
-    return 0.5f * z * (1.f + tanhf(C_GELU * (z + 0.044715f * z * z * z)));
-}
-__device__ __forceinline__ float gelu_grad(float z) {
-    const float t = tanhf(C_GELU * (z + 0.044715f * z * z * z));
-    return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * C_GELU * (1.f + 3.f * 0.044715f * z * z);
-}
 
 // Z += b (per column); A = gelu(Z) for hidden layers, A = Z for the output layer
 __global__ void k_bias_act(float *Z, float *A, const float *b, long long bz, int rows, int cols,
@@ -104,16 +72,9 @@ __global__ void k_colsum(const float *G, float *db, int rows, int cols, long lon
     db[z * sb + j] = s;
 }
 
-__global__ void k_adam(float *p, const float *g, float *m, float *v, long long n, float lr,
-                       float b1, float b2, float eps, float c1, float c2) {
+__global__ void k_adam(float *p, const float *g, float *m, float *v, long long n, AdamArgs a) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    if (i < n) adam_step(a, g[i], p[i], m[i], v[i]);
 }
 
 __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
@@ -125,12 +86,16 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 }
 
 // `rows` samples per member into the member's batch buffers (row stride mrows): drawn from
-// n with replacement (random = 1) or rows 0.. of X and T (random = 0)
+// n with replacement (random = 1) or rows 0.. of X and T (random = 0).  One thread a value:
+// one thread a row, looping over its 6 + 33 values, took 8.4 us for 5 x 128 rows.
 __global__ void k_gather(const float *X, const float *T, float *Xb, float *Tb, long long n, int rows,
                          int mrows, int din, int dout, unsigned long long seed, long long step,
                          int random) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const int z = blockIdx.y;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int z = blockIdx.y, w = din + dout;
+    const int r = (int)(i / w), k = (int)(i % w);
     if (r >= rows) return;
     long long s = r;
     if (random) {
@@ -139,22 +104,21 @@ __global__ void k_gather(const float *X, const float *T, float *Xb, float *Tb, l
         s = (long long)(h % (unsigned long long)n);
     }
     const long long o = (long long)z * mrows + r;
-    for (int k = 0; k < din; k++) Xb[o * din + k] = X[s * din + k];
-    for (int k = 0; k < dout; k++) Tb[o * dout + k] = T[s * dout + k];
+    if (k < din) Xb[o * din + k] = X[s * din + k];
+    else Tb[o * dout + k - din] = T[s * dout + k - din];
 }
 
-// rows of each member's output batch into Y (members x n x dout) at row offset c0
-__global__ void k_copy_out(const float *A, float *Y, int rows, int dout, int mrows, long long n,
-                           long long c0) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int z = blockIdx.y;
-    if (i >= (long long)rows * dout) return;
-    Y[((long long)z * n + c0) * dout + i] = A[(long long)z * mrows * dout + i];
-}
-
-__global__ void k_to_f32(const double *src, float *dst, long long n) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = (float)src[i];
+// the caller's parameters (members at stride cP, packed) into the padded layout
+__global__ void k_params_in(const double *src, float *dst, MlpOffsets from, MlpOffsets to, MlpOffsets len,
+                            int L, long long cP, long long P) {
+    const int z = blockIdx.y / L, l = blockIdx.y % L;
+    const double *s = src + z * cP;
+    float *d = dst + z * P;
+    for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < len.w[l] + len.b[l];
+         i += (long long)gridDim.x * blockDim.x) {
+        if (i < len.w[l]) d[to.w[l] + i] = (float)s[from.w[l] + i];
+        else d[to.b[l] + i - len.w[l]] = (float)s[from.b[l] + i - len.w[l]];
+    }
 }
 
 inline unsigned blocks(long long n, int b = 256) { return (unsigned)((n + b - 1) / b); }
@@ -168,18 +132,20 @@ struct MlpImpl {
     int E = 0, L = 0, max_batch = 0, maxw = 0;
     std::vector<int> sz;
     std::vector<long long> woff, boff;
-    long long P = 0;
+    long long P = 0, cP = 0;       // parameters of a member: stride here, the caller's count
+    MlpOffsets off{}, coff{}, len{};   // here, in the caller's arrays, and how many
     float *params = nullptr, *grads = nullptr, *am = nullptr, *av = nullptr, *Tb = nullptr,
           *loss = nullptr;
     double *stage = nullptr;
     std::vector<float *> act, pre;
-    float *gbuf[2] = {nullptr, nullptr};
+    float *gbuf[3] = {nullptr, nullptr, nullptr};
     long long adam_step = 0;
     MlpTc tc;               // BF16 tensor-core copy of the parameters
-    bool tc_dirty = true;   // parameters changed since it was packed
+    MlpF32 f32;             // packed FP32 copy of the parameters for whole-network inference
+    bool tc_dirty = true, f32_dirty = true;   // parameters changed since it was packed
     // training products on the tensor cores (pic_mlp_set_training): packed BF16 operand
     // scratch and the bounded-wait counter
-    bool train_tc = false, gemm_tc = false;
+    bool train_tc = false;
     uint16_t *tsa = nullptr, *tsb = nullptr;
     unsigned int *terr = nullptr;
 
@@ -206,6 +172,17 @@ struct MlpImpl {
         return PIC_OK;
     }
 
+    // places of arrays in one allocation
+    struct Carver {
+        std::vector<std::pair<void **, size_t>> at;
+        size_t bytes = 0;
+        template <class T>
+        void want(T *&p, long long n) {
+            at.push_back({reinterpret_cast<void **>(&p), bytes});
+            bytes += (sizeof(T) * (size_t)std::max<long long>(n, 1) + 255) / 256 * 256;
+        }
+    };
+
     pic_status init(int members, int layers, const int32_t *sizes, int batch) {
         E = members;
         L = layers;
@@ -213,24 +190,33 @@ struct MlpImpl {
         sz.assign(sizes, sizes + layers + 1);
         maxw = *std::max_element(sz.begin(), sz.end());
         for (int l = 0; l < L; l++) {
-            woff.push_back(P);
-            P += (long long)sz[l + 1] * sz[l];
-            boff.push_back(P);
-            P += sz[l + 1];
+            len.w[l] = (long long)sz[l + 1] * sz[l];
+            len.b[l] = sz[l + 1];
+            off.w[l] = P;
+            P += (len.w[l] + 3) / 4 * 4;
+            off.b[l] = P;
+            P += (len.b[l] + 3) / 4 * 4;
+            coff.w[l] = cP;
+            coff.b[l] = cP + len.w[l];
+            cP += len.w[l] + len.b[l];
+            woff.push_back(off.w[l]);
+            boff.push_back(off.b[l]);
         }
-        pic_status st;
-        if ((st = dalloc(params, E * P)) || (st = dalloc(grads, E * P)) || (st = dalloc(am, E * P)) ||
-            (st = dalloc(av, E * P)) || (st = dalloc(stage, E * P)) ||
-            (st = dalloc(Tb, (long long)E * batch * sz[L])) || (st = dalloc(loss, E)) ||
-            (st = dalloc(gbuf[0], (long long)E * batch * maxw)) ||
-            (st = dalloc(gbuf[1], (long long)E * batch * maxw)))
-            return st;
+        // everything in one allocation, each array on a 256-byte boundary
+        Carver carve;
+        carve.want(params, E * P);   // these four are cleared together
+        carve.want(grads, E * P);
+        carve.want(am, E * P);
+        carve.want(av, E * P);
+        const size_t cleared = carve.bytes;
+        carve.want(stage, E * cP);
+        carve.want(Tb, (long long)E * batch * sz[L]);
+        carve.want(loss, E);
+        for (float *&g : gbuf) carve.want(g, (long long)E * batch * maxw);
         act.assign(L + 1, nullptr);
         pre.assign(L, nullptr);
-        for (int l = 0; l <= L; l++)
-            if ((st = dalloc(act[l], (long long)E * batch * sz[l]))) return st;
-        for (int l = 0; l < L; l++)
-            if ((st = dalloc(pre[l], (long long)E * batch * sz[l + 1]))) return st;
+        for (int l = 0; l <= L; l++) carve.want(act[l], (long long)E * batch * sz[l]);
+        for (int l = 0; l < L; l++) carve.want(pre[l], (long long)E * batch * sz[l + 1]);
         // tensor-core inference: every width at most 256
         tc.ok = L <= MLP_MAX_LAYERS && maxw <= 256;
         if (tc.ok) {
@@ -246,18 +232,39 @@ struct MlpImpl {
                 tc.boff[l] = tc.bmember;
                 tc.bmember += tc.np[l];
             }
-            if ((st = dalloc(tc.w, E * tc.wmember)) || (st = dalloc(tc.b, E * tc.bmember)) ||
-                (st = dalloc(tc.err, 1)))
-                return st;
+            carve.want(tc.w, E * tc.wmember);
+            carve.want(tc.b, E * tc.bmember);
+            carve.want(tc.err, 1);
             const long long mp = (std::max(max_batch, maxw) + 127) / 128 * 128;
-            if ((st = dalloc(tsa, (long long)E * mp * 256)) ||
-                (st = dalloc(tsb, (long long)E * 256 * 256)) || (st = dalloc(terr, 1)))
-                return st;
-            PIC_CUDA_TRY(cudaMemset(terr, 0, sizeof(unsigned int)));
+            carve.want(tsa, (long long)E * mp * 256);
+            carve.want(tsb, (long long)E * 256 * 256);
+            carve.want(terr, 1);
         }
-        PIC_CUDA_TRY(cudaMemset(params, 0, sizeof(float) * E * P));
-        PIC_CUDA_TRY(cudaMemset(am, 0, sizeof(float) * E * P));
-        PIC_CUDA_TRY(cudaMemset(av, 0, sizeof(float) * E * P));
+        // whole-network FP32 inference: every width at most 256
+        f32.ok = maxw <= 256;
+        if (f32.ok) {
+            f32.E = E;
+            f32.L = L;
+            f32.NW = maxw <= 64 ? 64 : maxw <= 128 ? 128 : 256;
+            for (int l = 0; l < L; l++) {
+                f32.k[l] = sz[l];
+                f32.n[l] = sz[l + 1];
+                f32.kp[l] = (sz[l] + 15) / 16 * 16;
+                f32.np[l] = mlp_f32_shape(maxw, sz[l + 1]);
+                f32.woff[l] = f32.wmember;
+                f32.wmember += (long long)f32.kp[l] * f32.np[l];
+                f32.boff[l] = f32.bmember;
+                f32.bmember += f32.np[l];
+            }
+            carve.want(f32.w, E * f32.wmember);
+            carve.want(f32.b, E * f32.bmember);
+        }
+        unsigned char *base = nullptr;
+        pic_status st = dalloc(base, (long long)carve.bytes);
+        if (st != PIC_OK) return st;
+        for (const auto &x : carve.at) *x.first = base + x.second;
+        PIC_CUDA_TRY(cudaMemset(base, 0, cleared));
+        if (terr) PIC_CUDA_TRY(cudaMemset(terr, 0, sizeof(unsigned int)));
         return PIC_OK;
     }
 
@@ -276,17 +283,169 @@ struct MlpImpl {
         return PIC_OK;
     }
 
+    // one product of the tensor-core training path; its K may exceed what that takes
     void gemm(const GemmArgs &g, cudaStream_t s) {
-        if (gemm_tc) {
-            const TcGemmOp op{g.A, g.B, g.C, g.M, g.N, g.K, g.sAz, g.sBz, g.sCz,
-                              g.sAm, g.sAk, g.sBk, g.sBn, g.ldc, g.accumulate};
-            if (mlp_tc_gemm(op, E, tsa, tsb, terr, s)) return;
-        }
-        dim3 grid((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, E);
-        k_gemm<<<grid, dim3(GT, GT), 0, s>>>(g);
-        PIC_LAUNCHED();
+        const TcGemmOp op{g.A, g.B, g.C, g.M, g.N, g.K, g.sAz, g.sBz, g.sCz,
+                          g.sAm, g.sAk, g.sBk, g.sBn, g.ldc, g.accumulate};
+        if (mlp_tc_gemm(op, E, tsa, tsb, terr, s)) return;
+        MlpJobs jobs;
+        MlpJob &j = jobs.job[jobs.n++];
+        j = MlpJob{};
+        j.kind = g.sAm == 1 && g.sBn == 1 ? MLP_DW : g.sBn == 1 ? MLP_DX : MLP_FWD;
+        j.epi = MLP_EPI_STORE;
+        j.M = g.M;
+        j.N = g.N;
+        j.K = g.K;
+        j.A = g.A;
+        j.B = g.B;
+        j.C = g.C;
+        j.sA = g.sAz;
+        j.sB = g.sBz;
+        j.sC = g.sCz;
+        j.lda = j.kind == MLP_DW ? g.sAk : g.sAm;
+        j.ldb = j.kind == MLP_FWD ? g.sBn : g.sBk;
+        j.ldc = g.ldc;
+        mlp_jobs(jobs, E, s);
     }
 
+    // ---- the FP32 path: every product with what follows it (k_mlp_f32.cu) ----
+    // layer l for `rows` samples of A; C: where its outputs go (member stride sC)
+    MlpJob forward_job(int l, int rows, const float *A, long long sA, float *C, long long sC) {
+        MlpJob j{};
+        j.kind = MLP_FWD;
+        j.epi = l < L - 1 ? MLP_EPI_GELU : MLP_EPI_BIAS;
+        j.M = rows;
+        j.N = j.ldc = sz[l + 1];
+        j.K = j.lda = j.ldb = sz[l];
+        j.A = A;
+        j.sA = sA;
+        j.B = params + woff[l];
+        j.sB = j.sbias = P;
+        j.bias = params + boff[l];
+        j.C = C;
+        j.sC = sC;
+        return j;
+    }
+    // `rows` samples of X (every member the same) through all layers into Y (n rows a
+    // member), from row c0 on
+    void infer(int rows, const float *X, float *Y, long long n, long long c0, cudaStream_t s) {
+        const float *A = X;
+        long long sA = 0;
+        for (int l = 0; l < L; l++) {
+            const bool last = l == L - 1;
+            MlpJobs jobs;
+            jobs.job[jobs.n++] = forward_job(l, rows, A, sA, last ? Y + c0 * sz[L] : act[l + 1],
+                                             last ? n * sz[L] : (long long)max_batch * sz[l + 1]);
+            mlp_jobs(jobs, E, s);
+            A = act[l + 1];
+            sA = (long long)max_batch * sz[l + 1];
+        }
+    }
+    // the batch in act[0], Tb: losses (where asked for), gradients, and with `adam` the
+    // parameters' step in the place of the gradients' storing.  The weight gradients of a
+    // layer go with the next input gradient, which reads other weights.
+    void fused_step(int rows, float *loss_out, const AdamArgs *adam, cudaStream_t s) {
+        const long long sg = (long long)max_batch * maxw;
+        const auto sa = [&](int l) { return (long long)max_batch * sz[l]; };
+        for (int l = 0; l < L; l++) {
+            MlpJobs jobs;
+            const bool last = l == L - 1;
+            MlpJob &j = jobs.job[jobs.n++];
+            j = forward_job(l, rows, act[l], sa(l), last ? gbuf[l % 3] : act[l + 1], last ? sg : sa(l + 1));
+            if (last) {
+                j.epi = MLP_EPI_LOSS;
+                j.Z = Tb;
+                j.sZ = sa(L);
+                j.scale = 2.f / (float)((long long)rows * sz[L]);
+                j.loss = loss_out;
+            } else {
+                j.Z = pre[l];
+                j.sZ = sa(l + 1);
+            }
+            mlp_jobs(jobs, E, s);
+        }
+        const auto dx = [&](int l) {
+            MlpJob j{};
+            j.kind = MLP_DX;
+            j.epi = MLP_EPI_GELU_GRAD;
+            j.M = rows;
+            j.N = j.ldb = j.ldc = sz[l];
+            j.K = j.lda = sz[l + 1];
+            j.A = gbuf[l % 3];
+            j.sA = j.sC = sg;
+            j.B = params + woff[l];
+            j.sB = P;
+            j.C = gbuf[(l - 1) % 3];
+            j.Z = pre[l - 1];
+            j.sZ = sa(l);
+            return j;
+        };
+        const auto dw = [&](int l) {
+            MlpJob j{};
+            j.kind = MLP_DW;
+            j.M = j.lda = sz[l + 1];
+            j.N = j.ldb = j.ldc = sz[l];
+            j.K = rows;
+            j.A = gbuf[l % 3];
+            j.sA = sg;
+            j.B = act[l];
+            j.sB = sa(l);
+            j.sC = P;
+            if (adam) {
+                j.epi = MLP_EPI_ADAM;
+                j.adam = *adam;
+                j.C = params + woff[l];
+                j.am = am + woff[l];
+                j.av = av + woff[l];
+                j.db = params + boff[l];
+                j.dbm = am + boff[l];
+                j.dbv = av + boff[l];
+            } else {
+                j.epi = MLP_EPI_STORE;
+                j.C = grads + woff[l];
+                j.db = grads + boff[l];
+            }
+            return j;
+        };
+        for (int l = L - 1; l >= 1; l--) {
+            MlpJobs jobs;
+            jobs.job[jobs.n++] = dx(l);
+            if (l + 1 < L) jobs.job[jobs.n++] = dw(l + 1);
+            mlp_jobs(jobs, E, s);
+        }
+        MlpJobs jobs;
+        if (L > 1) jobs.job[jobs.n++] = dw(1);
+        jobs.job[jobs.n++] = dw(0);
+        mlp_jobs(jobs, E, s);
+    }
+
+    void gather(int rows, const float *X, const float *T, long long n, unsigned long long seed,
+                long long step, int random, cudaStream_t s) {
+        launch_chained(k_gather, dim3(blocks((long long)rows * (sz[0] + sz[L])), E), 256, 0, s, X, T, act[0],
+                       Tb, n, rows, max_batch, sz[0], sz[L], seed, step, random);
+    }
+    // FP32 inference on n rows by the whole-network kernel, or layer by layer in batches of
+    // max_batch.  A block of the whole-network kernel takes as long for one row as for its
+    // 64 to 256 (us for 6 -> 4 x 256 -> 33: 105, with 4 x 128: 64, with 4 x 64: 43), and
+    // 300 blocks run side by side; a batch of 256 rows layer by layer takes 49, 27 and 27 us
+    // for five members.  Measured, five members: 512 rows 105 / 64 / 43 against 97 / 52 / 38,
+    // 768 rows 105 / 64 / 43 against 145 / 78 / 54; one member of 4 x 256: 1024 rows 105
+    // against 101.
+    bool whole_network(long long n) const {
+        return f32.ok && n > std::min<long long>(2LL * max_batch, 1024);
+    }
+    // parameters changed: the packed copies are out of date
+    void touched() { tc_dirty = f32_dirty = true; }
+    // E x cP doubles from E x P floats
+    void unpad(const float *h, double *out) const {
+        for (int z = 0; z < E; z++)
+            for (int l = 0; l < L; l++) {
+                for (long long i = 0; i < len.w[l]; i++) out[z * cP + coff.w[l] + i] = h[z * P + off.w[l] + i];
+                for (long long i = 0; i < len.b[l]; i++) out[z * cP + coff.b[l] + i] = h[z * P + off.b[l] + i];
+            }
+    }
+
+    // ---- the tensor-core training path: products, then elementwise kernels ----
     // all layers for `rows` samples; the input of member z is X0 + z * sX0z (row-major)
     void forward(int rows, const float *X0, long long sX0z, cudaStream_t s) {
         const float *A = X0;
@@ -317,10 +476,11 @@ struct MlpImpl {
         // G is stored with the layer's width as row stride, member stride sg
         for (int l = L - 1; l >= 0; l--) {
             const int K = sz[l], N = sz[l + 1];
-            if (l < L - 1)
+            if (l < L - 1) {
                 k_gelu_back<<<dim3(blocks((long long)rows * N), E), 256, 0, s>>>(
                     G, pre[l], (long long)rows * N, sg, (long long)max_batch * N);
                 PIC_LAUNCHED();
+            }
             GemmArgs dw{G, act[l], grads + woff[l], N, K, rows, sg, (long long)max_batch * K, P,
                         1, N, K, 1, K, 0};
             gemm(dw, s);
@@ -389,7 +549,7 @@ extern "C" pic_status pic_mlp_param_count(pic_mlp *m, int64_t *per_member) try {
         set_error("pic_mlp_param_count: null output");
         return PIC_ERR_ARG;
     }
-    *per_member = m->impl->P;
+    *per_member = m->impl->cP;
     return PIC_OK;
 }
 PIC_CATCH("pic_mlp_param_count")
@@ -402,13 +562,13 @@ extern "C" pic_status pic_mlp_params_set(pic_mlp *m, const double *params) try {
         return PIC_ERR_ARG;
     }
     const long long n = x.E * x.P;
-    PIC_CUDA_TRY(cudaMemcpy(x.stage, params, sizeof(double) * n, cudaMemcpyHostToDevice));
-    k_to_f32<<<blocks(n), 256>>>(x.stage, x.params, n);
+    PIC_CUDA_TRY(cudaMemcpy(x.stage, params, sizeof(double) * x.E * x.cP, cudaMemcpyHostToDevice));
+    k_params_in<<<dim3(64, x.E * x.L), 256>>>(x.stage, x.params, x.coff, x.off, x.len, x.L, x.cP, x.P);
     PIC_LAUNCHED();
     PIC_CUDA_TRY(cudaMemset(x.am, 0, sizeof(float) * n));
     PIC_CUDA_TRY(cudaMemset(x.av, 0, sizeof(float) * n));
     x.adam_step = 0;
-    x.tc_dirty = true;
+    x.touched();
     PIC_CUDA_TRY(cudaDeviceSynchronize());
     return PIC_OK;
 }
@@ -424,7 +584,7 @@ extern "C" pic_status pic_mlp_params_get(pic_mlp *m, double *params) try {
     std::vector<float> h(x.E * x.P);
     PIC_CUDA_TRY(cudaDeviceSynchronize());
     PIC_CUDA_TRY(cudaMemcpy(h.data(), x.params, sizeof(float) * h.size(), cudaMemcpyDeviceToHost));
-    for (size_t i = 0; i < h.size(); i++) params[i] = h[i];
+    x.unpad(h.data(), params);
     return PIC_OK;
 }
 PIC_CATCH("pic_mlp_params_get")
@@ -439,14 +599,15 @@ extern "C" pic_status pic_mlp_grad(pic_mlp *m, const float *X, const float *T, i
     }
     cudaStream_t s = (cudaStream_t)st;
     const int rows = (int)n;
-    k_gather<<<dim3(blocks(rows), x.E), 256, 0, s>>>(X, T, x.act[0], x.Tb, n, rows, x.max_batch,
-                                                     x.sz[0], x.sz[x.L], 0, 0, 0);
-    PIC_LAUNCHED();
+    x.gather(rows, X, T, n, 0, 0, 0, s);
     PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
-    x.gemm_tc = x.train_tc;
-    x.forward(rows, x.act[0], (long long)x.max_batch * x.sz[0], s);
-    x.backward(rows, x.loss, s);
-    x.gemm_tc = false;
+    if (x.train_tc) {
+        x.forward(rows, x.act[0], (long long)x.max_batch * x.sz[0], s);
+        x.backward(rows, x.loss, s);
+    } else {
+        x.fused_step(rows, x.loss, nullptr, s);
+    }
+    PIC_CUDA_TRY(cudaGetLastError());
     pic_status ts = x.tc_errors("pic_mlp_grad", s);
     if (ts != PIC_OK) return ts;
     std::vector<float> h(x.E * x.P), hl(x.E);
@@ -454,7 +615,7 @@ extern "C" pic_status pic_mlp_grad(pic_mlp *m, const float *X, const float *T, i
                                  cudaMemcpyDeviceToHost, s));
     PIC_CUDA_TRY(cudaMemcpyAsync(hl.data(), x.loss, sizeof(float) * x.E, cudaMemcpyDeviceToHost, s));
     PIC_CUDA_TRY(cudaStreamSynchronize(s));
-    for (size_t i = 0; i < h.size(); i++) grads[i] = h[i];
+    x.unpad(h.data(), grads);
     if (loss)
         for (int z = 0; z < x.E; z++) loss[z] = hl[z];
     return PIC_OK;
@@ -472,26 +633,24 @@ extern "C" pic_status pic_mlp_train(pic_mlp *m, const float *X, const float *T, 
     }
     cudaStream_t s = (cudaStream_t)st;
     const long long np = x.E * x.P;
-    x.tc_dirty = true;
-    x.gemm_tc = x.train_tc;
+    x.touched();
     for (long long k = 0; k < steps; k++) {
-        k_gather<<<dim3(blocks(batch), x.E), 256, 0, s>>>(X, T, x.act[0], x.Tb, n, batch,
-                                                          x.max_batch, x.sz[0], x.sz[x.L], seed,
-                                                          x.adam_step, 1);
-        PIC_LAUNCHED();
+        x.gather(batch, X, T, n, seed, x.adam_step, 1, s);
         const bool last = k == steps - 1;
         if (last) PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
-        x.forward(batch, x.act[0], (long long)x.max_batch * x.sz[0], s);
-        x.backward(batch, last ? x.loss : nullptr, s);
         x.adam_step++;
         const float b1 = 0.9f, b2 = 0.999f;
-        const float c1 = 1.f - std::pow(b1, (float)x.adam_step);
-        const float c2 = 1.f - std::pow(b2, (float)x.adam_step);
-        k_adam<<<blocks(np), 256, 0, s>>>(x.params, x.grads, x.am, x.av, np, (float)lr, b1, b2,
-                                          1e-8f, c1, c2);
-        PIC_LAUNCHED();
+        const AdamArgs adam{(float)lr, b1, b2, 1e-8f, 1.f - std::pow(b1, (float)x.adam_step),
+                            1.f - std::pow(b2, (float)x.adam_step)};
+        if (x.train_tc) {
+            x.forward(batch, x.act[0], (long long)x.max_batch * x.sz[0], s);
+            x.backward(batch, last ? x.loss : nullptr, s);
+            k_adam<<<blocks(np), 256, 0, s>>>(x.params, x.grads, x.am, x.av, np, adam);
+            PIC_LAUNCHED();
+        } else {
+            x.fused_step(batch, last ? x.loss : nullptr, &adam, s);
+        }
     }
-    x.gemm_tc = false;
     PIC_CUDA_TRY(cudaGetLastError());
     pic_status ts = x.tc_errors("pic_mlp_train", s);
     if (ts != PIC_OK) return ts;
@@ -526,15 +685,17 @@ extern "C" pic_status pic_mlp_forward(pic_mlp *m, const float *X, float *Y, int6
         }
         return mlp_tc_forward(x.tc, X, Y, n, (cudaStream_t)st);
     }
+    if (n == 0) return PIC_OK;
     cudaStream_t s = (cudaStream_t)st;
-    const int din = x.sz[0], dout = x.sz[x.L];
-    for (long long c0 = 0; c0 < n; c0 += x.max_batch) {
-        const int rows = (int)std::min<long long>(x.max_batch, n - c0);
-        x.forward(rows, X + c0 * din, 0, s);
-        k_copy_out<<<dim3(blocks((long long)rows * dout), x.E), 256, 0, s>>>(
-            x.act[x.L], Y, rows, dout, x.max_batch, n, c0);
-        PIC_LAUNCHED();
+    if (x.whole_network(n)) {
+        if (x.f32_dirty) {
+            mlp_f32_pack(x.f32, x.params, x.P, x.off, s);
+            x.f32_dirty = false;
+        }
+        return mlp_f32_forward(x.f32, X, Y, n, s);
     }
+    for (long long c0 = 0; c0 < n; c0 += x.max_batch)
+        x.infer((int)std::min<long long>(x.max_batch, n - c0), X + c0 * x.sz[0], Y, n, c0, s);
     PIC_CUDA_TRY(cudaGetLastError());
     return PIC_OK;
 }

@@ -84,6 +84,66 @@ struct TcGemmOp {
 };
 bool mlp_tc_gemm(const TcGemmOp &g, int E, uint16_t *scratch_a, uint16_t *scratch_b,
                  unsigned int *err, cudaStream_t s);
+
+// ---- FP32 networks (k_mlp_f32.cu) ----
+// One product of a layer for every member, and what is done with each element of it.
+enum { MLP_FWD, MLP_DX, MLP_DW };   // A W^T, G W, G^T A
+enum {
+    MLP_EPI_STORE,      // C = x (DW: db = column sums of G, where db is set)
+    MLP_EPI_BIAS,       // v = x + bias; C = v (and Z = v, where Z is set)
+    MLP_EPI_GELU,       // the same with C = gelu(v)
+    // from here on Z or C is read:
+    MLP_EPI_LOSS,       // e = x + bias - Z; C = scale e; loss += e^2 / (M N), where loss is set
+    MLP_EPI_GELU_GRAD,  // C = x gelu'(Z)
+    MLP_EPI_ADAM,       // x is the gradient of C (am, av its moments), the column sums that of db
+};
+struct AdamArgs {
+    float lr, b1, b2, eps, c1, c2;   // c1, c2: the bias corrections of this step
+};
+struct MlpJob {
+    int kind, epi;
+    int M, N, K;
+    const float *A, *B;         // lda, ldb: stride of the index the operand is not contiguous along
+    float *C;
+    long long sA, sB, sC;       // member strides; db's is sC
+    int lda, ldb, ldc;
+    const float *bias;
+    float *Z;                   // laid out like C, member stride sZ
+    long long sbias, sZ;
+    float *db, *am, *av, *dbm, *dbv;
+    float scale;
+    float *loss;
+    AdamArgs adam;
+};
+constexpr int MLP_MAX_JOBS = 3;
+struct MlpJobs {
+    MlpJob job[MLP_MAX_JOBS];   // in the order that the blocks take them
+    int blocks[MLP_MAX_JOBS];
+    int n = 0;
+};
+// the jobs in one launch (their results must not depend on each other)
+void mlp_jobs(MlpJobs &jobs, int E, cudaStream_t s);
+
+// Parameters as the whole-network kernel reads them: per member and layer the weights
+// k-major (kp x np: kp the inputs up to a multiple of 16, np by mlp_f32_shape) and np biases.
+struct MlpF32 {
+    int E = 0, L = 0, NW = 0;                              // NW: 64, 128 or 256 units at most
+    int k[MLP_MAX_LAYERS] = {}, n[MLP_MAX_LAYERS] = {};
+    int kp[MLP_MAX_LAYERS] = {}, np[MLP_MAX_LAYERS] = {};
+    long long woff[MLP_MAX_LAYERS] = {}, boff[MLP_MAX_LAYERS] = {};
+    long long wmember = 0, bmember = 0;
+    float *w = nullptr, *b = nullptr;
+    bool ok = false;
+};
+struct MlpOffsets {
+    long long w[MLP_MAX_LAYERS], b[MLP_MAX_LAYERS];        // in a member's parameters
+};
+int mlp_f32_shape(int maxw, int width);
+void mlp_f32_pack(const MlpF32 &net, const float *params, long long P, const MlpOffsets &o,
+                  cudaStream_t s);
+// Y (E x n x outputs) from X (n x inputs)
+pic_status mlp_f32_forward(const MlpF32 &net, const float *X, float *Y, int64_t n, cudaStream_t s);
+
 #define PIC_CUDA_TRY(expr)                                                              \
     do {                                                                                \
         cudaError_t err__ = (expr);                                                     \
@@ -184,6 +244,28 @@ bool build_emit_line(const HostMesh &m, double z0, double rho0, double rho1,
 void note_launches(long long k);
 long long launches_this_thread();
 #define PIC_LAUNCHED() ::pic::note_launches(1)
+
+// Launch of a kernel of a dependent chain: its blocks may take their places while the
+// kernel before it drains, and wait there (griddepcontrol.wait, the kernel's first
+// statement) until that one has completed and its writes are visible.  The kernel lets its
+// own successor in the same way right after its wait (griddepcontrol.launch_dependents),
+// so that whatever a kernel has waited for has completed before its successor starts.
+template <class... Params, class... Args>
+void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                    Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    PIC_LAUNCHED();
+}
 
 // ---------------------------------------------------------------------------------
 // device layouts
