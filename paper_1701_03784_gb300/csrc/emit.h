@@ -1,14 +1,20 @@
-// Cathode emission (Secs. 5.2, 5.3: electrons leave the cathode every step).  One block
-// appends per_step particles behind the live slots at the start of a step, before the
-// particle kernel: positions on the line z = const, uniform in area over [rho0, rho1];
+// Cathode emission (Secs. 5.2, 5.3: electrons leave the cathode every step), done by extra
+// blocks of the face kernel: they append per_step particles behind the live slots at the
+// start of a step, positions on the line z = const, uniform in area over [rho0, rho1];
 // momenta u = gamma v with normal components of spread u_thermal about (0, 0, u_normal).
 // Their charge (Eq. charge at the birth point) is added to Q^n, so that Eq. DCE holds for
 // the step, and taken out of the Gauss-law bookkeeping (it appears without a current).
+// None of this meets what the face kernel reads or writes, so the two run side by side.
 //
 // Draws are counter-based: for particle id p and draw j, splitmix64(seed + 8 p + j)
 // (the output function of Steele, Lea and Flood's generator, as Vigna publishes it), as a
 // double in (0, 1); Box-Muller on draws 1, 2 and 3, 4.
-#include <cmath>
+//
+// Bound by the FP64 units, two lanes a clock and SM: 2000 births in one block took 127 us
+// of a diode step (FP64 pipe 83% busy on that one SM).  A birth a thread over as many
+// blocks as that takes, and no thermal draws when the spread is zero, put them beside the
+// face kernel's 4 us.
+#pragma once
 
 #include "pic_internal.h"
 
@@ -28,27 +34,23 @@ __device__ __forceinline__ double unit_draw(unsigned long long seed, long long p
     return ((double)(splitmix64(x) >> 11) + 0.5) * 0x1.0p-53;
 }
 
-constexpr int EMIT_THREADS = 256;
-
+// Block b of nb blocks.  Every block reads the counts before it takes its ticket; the last
+// one to finish moves them on.
 template <class P>
-__global__ void __launch_bounds__(EMIT_THREADS) k_emit(EmitArgs<P> a) {
+__device__ __forceinline__ void emit_block(const EmitArgs<P> &a, int b, int nb) {
     __shared__ long long base_slot, base_pid;
-    __shared__ int room;
     if (threadIdx.x == 0) {
         base_slot = *a.n_slots;
         base_pid = (long long)a.counters[CNT_NEXT_PID];
-        room = base_slot + a.per_step <= a.cap;
-        if (!room) atomicAdd(a.counters + CNT_EMIT_DROPPED, (unsigned long long)a.per_step);
     }
     __syncthreads();
-    if (!room) return;
+    const bool room = base_slot + a.per_step <= a.cap;
     const double two_pi = 6.283185307179586476925286766559;
-    for (long long k = threadIdx.x; k < a.per_step; k += EMIT_THREADS) {
+    for (long long k = (long long)b * blockDim.x + threadIdx.x; room && k < a.per_step;
+         k += (long long)nb * blockDim.x) {
         const long long pid = base_pid + k;
-        double u[5];
-#pragma unroll
-        for (int j = 0; j < 5; j++) u[j] = unit_draw(a.seed, pid, j);
-        const double rho = sqrt(a.rho0 * a.rho0 + u[0] * (a.rho1 * a.rho1 - a.rho0 * a.rho0));
+        const double u0 = unit_draw(a.seed, pid, 0);
+        const double rho = sqrt(a.rho0 * a.rho0 + u0 * (a.rho1 * a.rho1 - a.rho0 * a.rho0));
         // the interval of the emission line that holds rho (intervals sorted and contiguous)
         int lo = 0, hi = a.line.n - 1;
         while (lo < hi) {
@@ -65,10 +67,16 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(EmitArgs<P> a) {
             lam[m] = fmax(la + s * (lb - la), 0.0);
         }
         const int t = a.line.tri[lo];
-        const double r1 = sqrt(-2.0 * log(u[1])), r3 = sqrt(-2.0 * log(u[3]));
-        const double ur = a.u_thermal * r1 * cos(two_pi * u[2]);
-        const double up = a.u_thermal * r1 * sin(two_pi * u[2]);
-        const double uz = a.u_normal + a.u_thermal * r3 * cos(two_pi * u[4]);
+        double ur = 0.0, up = 0.0, uz = a.u_normal;
+        if (a.u_thermal != 0.0) {
+            double u[5];
+#pragma unroll
+            for (int j = 1; j < 5; j++) u[j] = unit_draw(a.seed, pid, j);
+            const double r1 = sqrt(-2.0 * log(u[1])), r3 = sqrt(-2.0 * log(u[3]));
+            ur = a.u_thermal * r1 * cos(two_pi * u[2]);
+            up = a.u_thermal * r1 * sin(two_pi * u[2]);
+            uz = a.u_normal + a.u_thermal * r3 * cos(two_pi * u[4]);
+        }
         const long long i = base_slot + k;
         a.p.tri[i] = t;
         a.p.ur[i] = (typename P::R)ur;
@@ -109,22 +117,20 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_emit(EmitArgs<P> a) {
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        *a.n_slots = base_slot + a.per_step;
-        a.counters[CNT_EMITTED] += (unsigned long long)a.per_step;
-        a.counters[CNT_NEXT_PID] += (unsigned long long)a.per_step;
+        __threadfence();
+        if (atomicAdd(a.counters + CNT_EMIT_TICKET, 1ULL) == (unsigned long long)(nb - 1)) {
+            a.counters[CNT_EMIT_TICKET] = 0;
+            if (room) {
+                *a.n_slots = base_slot + a.per_step;
+                a.counters[CNT_EMITTED] += (unsigned long long)a.per_step;
+                a.counters[CNT_NEXT_PID] += (unsigned long long)a.per_step;
+            } else {
+                a.counters[CNT_EMIT_DROPPED] += (unsigned long long)a.per_step;
+            }
+        }
     }
 }
 
 }  // namespace
-
-template <class P>
-void launch_emit(const EmitArgs<P> &a, cudaStream_t s) {
-    if (a.per_step <= 0 || a.line.n <= 0) return;
-    k_emit<P><<<1, EMIT_THREADS, 0, s>>>(a);
-    PIC_LAUNCHED();
-}
-
-template void launch_emit<PF32>(const EmitArgs<PF32> &, cudaStream_t);
-template void launch_emit<PF64>(const EmitArgs<PF64> &, cudaStream_t);
 
 }  // namespace pic

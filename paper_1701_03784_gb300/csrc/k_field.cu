@@ -1,10 +1,23 @@
 // Field update of the mixed E-B leapfrog (Eqs. full_d_dfl, full_d_dal) and the per-step
 // triangle field records read by the particle kernel.
 #include <algorithm>
+#include <type_traits>
 
+#include "emit.h"
 #include "pic_internal.h"
+#include "record.h"
 
 namespace pic {
+
+// The kernels of a step are chained (launch_chained): a kernel's blocks take their places
+// while the one before it drains, load what never changes after creation (geometry,
+// incidence, matrix entries), wait, and only then touch anything that a kernel writes.
+// Measured with graph replay on 2000 triangles and 10,000 particles (FP64): 12.8 -> 9.5 us
+// a step; 32 steps enqueued one by one on 47k triangles and 500k particles: 1824 -> 1737 us.
+
+// s flipped where the edge runs against the counter-clockwise boundary
+template <class R>
+__device__ __forceinline__ R along(R e, bool fwd) { return fwd ? e : -e; }
 
 // K3, one thread per face: B^{n+1/2} = B^{n-1/2} - dt (D_curl E^n)_f, and the record's
 // field coefficients: E(lambda) = sum_k E_k (lambda_a grad lambda_b - lambda_b grad
@@ -13,86 +26,76 @@ namespace pic {
 // B_phi = (B^{n+1/2} + B^{n-1/2}) / (2A) (W2 = 1/A).  In a lossy layer
 // B^{n+1/2} = a_f B^{n-1/2} - b_f dt (D_curl E^n)_f.
 // The same launch clears the step's accumulators (J per edge, Q_abs per node, and in the
-// FP64 build Q^{n+1}, which the particle kernel accumulates).
-template <class P, bool STATIC, bool LOSS>
-__global__ void __launch_bounds__(512) k_field_b(FieldArgs<P> a) {
+// FP64 build Q^{n+1}, which the particle kernel accumulates).  Its first emit_blocks blocks
+// make the step's births (emit.h).
+// The record is read and written in 16-byte words (g | rho, 1/A | c0 c1 c2, B_phi, pad |
+// nodes, flags | edges, flags); in 8-byte ones the FP64 build's stores alone kept a launch
+// on 199k faces at 27 us.
+template <class P, bool STATIC, bool LOSS, bool EMIT>
+__global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldArgs<P> a,
+                                                 const __grid_constant__ EmitArgs<P> em, int emit_blocks) {
     using R = typename P::R;
-    int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    using R4 = typename std::conditional<sizeof(R) == 4, float4, double2>::type;   // 16 bytes
+    constexpr int W = 16 / sizeof(R);
+    if constexpr (EMIT) {
+        if ((int)blockIdx.x < emit_blocks) {
+            chain_wait();
+            emit_block<P>(em, blockIdx.x, emit_blocks);
+            return;
+        }
+    }
+    const int64_t f = (int64_t)(blockIdx.x - (EMIT ? emit_blocks : 0)) * blockDim.x + threadIdx.x;
+    const bool face = f < a.N2;
+    R g[2][2] = {}, inv_area = 0;
+    int4 EG = make_int4(0, 0, 0, 0);
+    if (face) {
+        const R *rc = reinterpret_cast<const R *>(a.rec + f);
+        R w[8];   // g (4), rho (3), 1/A
+#pragma unroll
+        for (int k = 0; k < 8; k += W) *reinterpret_cast<R4 *>(w + k) = *reinterpret_cast<const R4 *>(rc + k);
+        g[0][0] = w[0];
+        g[0][1] = w[1];
+        g[1][0] = w[2];
+        g[1][1] = w[3];
+        inv_area = w[7];
+        EG = *reinterpret_cast<const int4 *>(a.rec[f].edge);
+    }
+    chain_wait();
     if (f < a.N1) a.J[f] = 0;
     if (f < a.N0) {
         a.Qabs[f] = 0;
         if constexpr (!P::fixed) a.Qnext[f] = 0;
     }
-    if (f >= a.N2) return;
-    if constexpr (sizeof(R) == 4) {
-        // FP32 record: 16-byte groups (g | rho, 1/A | c0 c1 | c2, B_phi, pad | nodes, flags |
-        // edges, flags), read and written as vectors
-        float4 *R4 = reinterpret_cast<float4 *>(a.rec + f);
-        const float4 G = R4[0], RH = R4[1];
-        const int4 EG = reinterpret_cast<const int4 *>(a.rec + f)[5];
-        const float g[3][2] = {{G.x, G.y}, {G.z, G.w}, {-G.x - G.z, -G.y - G.w}};
-        float c[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-        float curl = 0;
-        const int ek[3] = {EG.x, EG.y, EG.z};
-        float E3[3], S3[3] = {0.f, 0.f, 0.f};
+    if (!face) return;
+    // edge values along the counter-clockwise boundary (edge k: local node k+1 -> k+2)
+    const int e3[3] = {EG.x, EG.y, EG.z};
+    R E3[3], s[3];
 #pragma unroll
-        for (int k = 0; k < 3; k++) E3[k] = a.E[ek[k]];
-        if constexpr (STATIC) {
-#pragma unroll
-            for (int k = 0; k < 3; k++) S3[k] = a.Es[ek[k]];
-        }
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const float Ek = STATIC ? E3[k] + S3[k] : E3[k];   // the gather sees the static field
-            const int i = (k + 1) % 3, j = (k + 2) % 3;
-            const bool fwd = (EG.w >> k) & 1;
-            const int ta = fwd ? i : j, hb = fwd ? j : i;
-            c[ta][0] += Ek * g[hb][0];
-            c[ta][1] += Ek * g[hb][1];
-            c[hb][0] -= Ek * g[ta][0];
-            c[hb][1] -= Ek * g[ta][1];
-            curl += fwd ? E3[k] : -E3[k];
-        }
-        const float Bold = a.B[f];
-        float Bnew = Bold - a.dt * curl;
-        if constexpr (LOSS) {
-            const float2 lf = reinterpret_cast<const float2 *>(a.loss_f)[f];
-            Bnew = lf.x * Bold - lf.y * (a.dt * curl);
-        }
-        a.B[f] = Bnew;
-        R4[2] = make_float4(c[0][0], c[0][1], c[1][0], c[1][1]);
-        R4[3] = make_float4(c[2][0], c[2][1], 0.5f * (Bnew + Bold) * RH.w, 0.f);
-        return;
-    }
-    TriRec<R> &rc = a.rec[f];
-    const int32_t flags = rc.flags;
-    R g[3][2] = {{rc.g[0], rc.g[1]}, {rc.g[2], rc.g[3]}, {-rc.g[0] - rc.g[2], -rc.g[1] - rc.g[3]}};
-    R c[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-    R curl = 0;
+    for (int k = 0; k < 3; k++) E3[k] = a.E[e3[k]];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const R Ed = a.E[rc.edge[k]];
-        R Ek = Ed;
-        if constexpr (STATIC) Ek += a.Es[rc.edge[k]];   // the gather sees the static field
-        int i = (k + 1) % 3, j = (k + 2) % 3;
-        bool fwd = (flags >> k) & 1;   // edge runs (k+1) -> (k+2): D_curl entry +1
-        int ta = fwd ? i : j, hb = fwd ? j : i;
-        c[ta][0] += Ek * g[hb][0];
-        c[ta][1] += Ek * g[hb][1];
-        c[hb][0] -= Ek * g[ta][0];
-        c[hb][1] -= Ek * g[ta][1];
-        curl += fwd ? Ed : -Ed;
+        const bool fwd = (EG.w >> k) & 1;
+        s[k] = along<R>(STATIC ? E3[k] + a.Es[e3[k]] : E3[k], fwd);   // the gather sees the static field
+        E3[k] = along<R>(E3[k], fwd);
     }
-    R Bold = a.B[f];
+    const R Bold = a.B[f];
+    const R curl = (E3[0] + E3[1]) + E3[2];
     R Bnew = Bold - a.dt * curl;
     if constexpr (LOSS) Bnew = a.loss_f[2 * f] * Bold - a.loss_f[2 * f + 1] * (a.dt * curl);
     a.B[f] = Bnew;
-    rc.bphi = R(0.5) * (Bnew + Bold) * rc.inv_area;
+    R w[8];
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        rc.c[2 * k] = c[k][0];
-        rc.c[2 * k + 1] = c[k][1];
+    for (int d = 0; d < 2; d++) {
+        const R g0 = g[0][d], g1 = g[1][d], g2 = -g0 - g1;
+        w[d] = fma(s[2], g1, -(s[1] * g2));
+        w[2 + d] = fma(-s[2], g0, s[0] * g2);
+        w[4 + d] = fma(s[1], g0, -(s[0] * g1));
     }
+    w[6] = R(0.5) * (Bnew + Bold) * inv_area;
+    w[7] = 0;
+    R *out = reinterpret_cast<R *>(a.rec + f) + 8;
+#pragma unroll
+    for (int k = 0; k < 8; k += W) *reinterpret_cast<R4 *>(out + k) = *reinterpret_cast<R4 *>(w + k);
 }
 
 // Per node, after the particle step.  FP32 build: Q^{n+1} = Q^n - (D_div J)/2^22 -
@@ -115,22 +118,46 @@ __device__ __forceinline__ void node_update(const FieldArgs<P> &a, int64_t k) {
 }
 
 // K4a, one thread per free edge: r = D_curl^T star_mu^-1 B^{n+1/2} - J^{n+1/2}; the DGL
-// auxiliary flux D += dt r.  The same launch does the per-node update (thread k, node k).
-template <class P>
-__global__ void __launch_bounds__(512) k_field_r(FieldArgs<P> a) {
+// auxiliary flux D += dt r.  The same launch does the per-node update (thread k, node k),
+// and its first blocks record probes and ports (record.h).
+template <class P, bool REC>
+__global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldArgs<P> a,
+                                                 const __grid_constant__ ProbeArgs<P> probe,
+                                                 const __grid_constant__ PortArgs<P> port) {
     using R = typename P::R;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int blk = blockIdx.x;
+    if constexpr (REC) {
+        if (blk < probe.n_groups + port.n_ports) {
+            chain_wait();
+            if (blk < probe.n_groups) probe_block<P>(probe, blk);
+            else port_block<P>(port, blk - probe.n_groups);
+            return;
+        }
+        blk -= probe.n_groups + port.n_ports;
+    }
+    const int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
+    int32_t e = 0;
+    int2 ef = make_int2(0, 0);
+    if (i < a.nf) {
+        e = a.free_edges[i];
+        ef = reinterpret_cast<const int2 *>(a.edge_face)[i];
+    }
+    R mu[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int32_t fs = q == 0 ? ef.x : ef.y;
+        if (fs != 0) mu[q] = a.mu_inv[(fs > 0 ? fs : -fs) - 1];
+    }
+    chain_wait();
     if (i < a.N0) node_update<P>(a, i);
     if (i >= a.nf) return;
-    const int32_t e = a.free_edges[i];
-    const int2 ef = reinterpret_cast<const int2 *>(a.edge_face)[i];
     double r = 0;
 #pragma unroll
     for (int q = 0; q < 2; q++) {
         int32_t fs = q == 0 ? ef.x : ef.y;
         if (fs == 0) continue;
         int32_t f = (fs > 0 ? fs : -fs) - 1;
-        double hf = (double)a.mu_inv[f] * (double)a.B[f];
+        double hf = (double)mu[q] * (double)a.B[f];
         r += fs > 0 ? hf : -hf;
     }
     double Jp;
@@ -145,74 +172,109 @@ __global__ void __launch_bounds__(512) k_field_r(FieldArgs<P> a) {
 // E_e <- a_e E_e + b_e dt (M r)_i, a = (1 - s)/(1 + s), b = 1/(1 + s), s = sigma dt/(2 eps0)).  A warp owns a slice of 32 rows
 // stored column-major, so each step of the row loop reads 32 consecutive values.
 template <class P, bool LOSS>
-__global__ void __launch_bounds__(512) k_field_spmv(FieldArgs<P> a) {
+__global__ void __launch_bounds__(512) k_field_spmv(const __grid_constant__ FieldArgs<P> a) {
     using R = typename P::R;
     int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t slice = row >> 5;
     int lane = (int)(row & 31);
     int64_t n_slices = (a.nf + 31) >> 5;
-    if (slice >= n_slices) return;
-    int64_t off = a.ell_off[slice];
-    int width = (int)((a.ell_off[slice + 1] - off) >> 5);
+    if (slice >= n_slices) {
+        chain_wait();
+        return;
+    }
+    const int64_t off = a.ell_off[slice];
+    const int width = (int)((a.ell_off[slice + 1] - off) >> 5);
+    const int32_t *cols = a.ell_col + off + lane;
+    const R *vals = a.ell_val + off + lane;
+    // HEAD columns' indices and values are in flight before the wait, four at a time after
+    // (the sum keeps the column order).  More of them ahead cost occupancy: 12 take 78
+    // registers, and 32 steps of the 200k-triangle BWO 12.14 ms; 8 12.03 ms; 4 11.98 ms
+    constexpr int HEAD = 4;
+    int32_t col[HEAD];
+    R val[HEAD];
+#pragma unroll
+    for (int u = 0; u < HEAD; u++)
+        if (u < width) {
+            col[u] = cols[u * 32];
+            val[u] = vals[u * 32];
+        }
+    const int32_t e = row < a.nf ? a.free_edges[row] : 0;
+    chain_wait();
     R acc = 0;
-    int k = 0;
-    // four columns' indices and values in flight before their gathers (the sum keeps the
-    // column order)
+    {
+        R rv[HEAD];
+#pragma unroll
+        for (int u = 0; u < HEAD; u++)
+            if (u < width) rv[u] = a.r[col[u]];
+#pragma unroll
+        for (int u = 0; u < HEAD; u++)
+            if (u < width) acc += val[u] * rv[u];
+    }
+    int k = HEAD;
     for (; k + 4 <= width; k += 4) {
-        int32_t col[4];
-        R val[4];
+        int32_t c4[4];
+        R v4[4], r4[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const int64_t idx = off + ((int64_t)(k + u) << 5) + lane;
-            col[u] = a.ell_col[idx];
-            val[u] = a.ell_val[idx];
+            c4[u] = cols[(int64_t)(k + u) * 32];
+            v4[u] = vals[(int64_t)(k + u) * 32];
         }
-        R rv[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) rv[u] = a.r[col[u]];
+        for (int u = 0; u < 4; u++) r4[u] = a.r[c4[u]];
 #pragma unroll
-        for (int u = 0; u < 4; u++) acc += val[u] * rv[u];
+        for (int u = 0; u < 4; u++) acc += v4[u] * r4[u];
     }
-    for (; k < width; k++) {
-        const int64_t idx = off + ((int64_t)k << 5) + lane;
-        acc += a.ell_val[idx] * a.r[a.ell_col[idx]];
-    }
+    for (; k < width; k++) acc += vals[(int64_t)k * 32] * a.r[cols[(int64_t)k * 32]];
     if (row < a.nf) {
-        const int32_t e = a.free_edges[row];
         if constexpr (LOSS) a.E[e] = a.loss_e[2 * row] * a.E[e] + a.loss_e[2 * row + 1] * (a.dt * acc);
         else a.E[e] += a.dt * acc;
     }
 }
 
 template <class P>
-void launch_field_b(const FieldArgs<P> &a, cudaStream_t s) {
+void launch_field_b(const FieldArgs<P> &a, const EmitArgs<P> *emit, cudaStream_t s) {
     const int64_t n = std::max(a.N2, std::max(a.N1, a.N0));
     const int b = a.block;
-    const unsigned g = (unsigned)((n + b - 1) / b);
-    // the optional static field and lossy layer as instantiations: none costs the common
-    // case anything
-    if (a.Es && a.loss_f) k_field_b<P, true, true><<<g, b, 0, s>>>(a);
-    else if (a.Es) k_field_b<P, true, false><<<g, b, 0, s>>>(a);
-    else if (a.loss_f) k_field_b<P, false, true><<<g, b, 0, s>>>(a);
-    else k_field_b<P, false, false><<<g, b, 0, s>>>(a);
-    PIC_LAUNCHED();
+    const bool births = emit && emit->per_step > 0 && emit->line.n > 0;
+    const EmitArgs<P> em = births ? *emit : EmitArgs<P>{};
+    // a birth a thread, up to one block an SM or so: beyond that the threads take several
+    const int eb = births ? (int)std::min<int64_t>((em.per_step + b - 1) / b, 1024) : 0;
+    const unsigned g = (unsigned)((n + b - 1) / b + eb);
+    // the optional static field, lossy layer and emission as instantiations: none costs the
+    // common case anything
+    const auto go = [&](auto kernel) { launch_chained(a.chain, kernel, g, b, 0, s, a, em, eb); };
+    if (births) {
+        if (a.Es && a.loss_f) go(k_field_b<P, true, true, true>);
+        else if (a.Es) go(k_field_b<P, true, false, true>);
+        else if (a.loss_f) go(k_field_b<P, false, true, true>);
+        else go(k_field_b<P, false, false, true>);
+    } else {
+        if (a.Es && a.loss_f) go(k_field_b<P, true, true, false>);
+        else if (a.Es) go(k_field_b<P, true, false, false>);
+        else if (a.loss_f) go(k_field_b<P, false, true, false>);
+        else go(k_field_b<P, false, false, false>);
+    }
 }
 
 template <class P>
-void launch_field_e(const FieldArgs<P> &a, cudaStream_t s) {
+void launch_field_e(const FieldArgs<P> &a, const ProbeArgs<P> &probe, const PortArgs<P> &port,
+                    cudaStream_t s) {
     const int64_t n = std::max(a.nf, a.N0);
-    const int b = a.block;
-    k_field_r<P><<<(unsigned)((n + b - 1) / b), b, 0, s>>>(a);
-    PIC_LAUNCHED();
+    const int b = a.block, nr = probe.n_groups + port.n_ports;
+    const unsigned g = (unsigned)((n + b - 1) / b + nr);
+    if (nr > 0) launch_chained(true, k_field_r<P, true>, g, b, 0, s, a, probe, port);
+    else launch_chained(true, k_field_r<P, false>, g, b, 0, s, a, probe, port);
     int64_t rows = ((a.nf + 31) / 32) * 32;
-    if (a.loss_e) k_field_spmv<P, true><<<(unsigned)((rows + b - 1) / b), b, 0, s>>>(a);
-    else k_field_spmv<P, false><<<(unsigned)((rows + b - 1) / b), b, 0, s>>>(a);
-    PIC_LAUNCHED();
+    const unsigned gs = (unsigned)((rows + b - 1) / b);
+    if (a.loss_e) launch_chained(true, k_field_spmv<P, true>, gs, b, 0, s, a);
+    else launch_chained(true, k_field_spmv<P, false>, gs, b, 0, s, a);
 }
 
-template void launch_field_b<PF32>(const FieldArgs<PF32> &, cudaStream_t);
-template void launch_field_b<PF64>(const FieldArgs<PF64> &, cudaStream_t);
-template void launch_field_e<PF32>(const FieldArgs<PF32> &, cudaStream_t);
-template void launch_field_e<PF64>(const FieldArgs<PF64> &, cudaStream_t);
+template void launch_field_b<PF32>(const FieldArgs<PF32> &, const EmitArgs<PF32> *, cudaStream_t);
+template void launch_field_b<PF64>(const FieldArgs<PF64> &, const EmitArgs<PF64> *, cudaStream_t);
+template void launch_field_e<PF32>(const FieldArgs<PF32> &, const ProbeArgs<PF32> &, const PortArgs<PF32> &,
+                                   cudaStream_t);
+template void launch_field_e<PF64>(const FieldArgs<PF64> &, const ProbeArgs<PF64> &, const PortArgs<PF64> &,
+                                   cudaStream_t);
 
 }  // namespace pic

@@ -231,8 +231,7 @@ __global__ void __launch_bounds__(Shape<T>::NT, 3) k_mlp_jobs(const __grid_const
     using S = Shape<T>;
     extern __shared__ __align__(16) unsigned char raw[];
     TileSmem<T> &sm = *reinterpret_cast<TileSmem<T> *>(raw);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_wait();
     int j = 0, blk = blockIdx.x;
     while (j + 1 < jobs.n && blk >= jobs.blocks[j]) blk -= jobs.blocks[j++];
     const MlpJob &g = jobs.job[j];
@@ -538,7 +537,7 @@ pic_status launch_fused(const MlpF32 &net, const float *X, float *Y, int64_t n, 
 }  // namespace
 
 template <int T>
-static void launch_jobs(const MlpJobs &jobs, unsigned blocks, cudaStream_t s) {
+static void launch_jobs(const MlpJobs &jobs, unsigned blocks, bool chain, cudaStream_t s) {
     const int smem = (int)sizeof(TileSmem<T>);
     static bool attr[64] = {};   // the shared-memory opt-in, once per device
     int dev = 0;
@@ -547,7 +546,7 @@ static void launch_jobs(const MlpJobs &jobs, unsigned blocks, cudaStream_t s) {
         cudaFuncSetAttribute(k_mlp_jobs<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         attr[dev & 63] = true;
     }
-    launch_chained(k_mlp_jobs<T>, blocks, Shape<T>::NT, smem, s, jobs);
+    launch_chained(chain, k_mlp_jobs<T>, blocks, Shape<T>::NT, smem, s, jobs);
 }
 
 int mlp_f32_shape(int maxw, int width) {
@@ -567,7 +566,7 @@ pic_status mlp_f32_forward(const MlpF32 &net, const float *X, float *Y, int64_t 
     return launch_fused<256>(net, X, Y, n, s);
 }
 
-void mlp_jobs(MlpJobs &jobs, int E, cudaStream_t s) {
+void mlp_jobs(MlpJobs &jobs, int E, bool chain, cudaStream_t s) {
     long long big = 0;
     for (int j = 0; j < jobs.n; j++)
         big += (long long)((jobs.job[j].M + 63) / 64) * ((jobs.job[j].N + 63) / 64) * E;
@@ -577,8 +576,8 @@ void mlp_jobs(MlpJobs &jobs, int E, cudaStream_t s) {
         jobs.blocks[j] = (int)((long long)((jobs.job[j].M + T - 1) / T) * ((jobs.job[j].N + T - 1) / T) * E);
         blocks += jobs.blocks[j];
     }
-    if (T == 64) launch_jobs<64>(jobs, (unsigned)blocks, s);
-    else launch_jobs<32>(jobs, (unsigned)blocks, s);
+    if (T == 64) launch_jobs<64>(jobs, (unsigned)blocks, chain, s);
+    else launch_jobs<32>(jobs, (unsigned)blocks, chain, s);
 }
 
 }  // namespace pic

@@ -173,7 +173,8 @@ __device__ __forceinline__ void load_bary<PF64>(const Particles<PF64> &p, int64_
 }  // namespace
 
 template <class P>
-__global__ void __launch_bounds__(256) k_push(PushArgs<P> a) {
+__global__ void __launch_bounds__(256) k_push(const __grid_constant__ PushArgs<P> a) {
+    chain_wait();
     using R = typename P::R;
     using Acc = typename P::Acc;
     using Contrib = typename std::conditional<P::fixed, long long, double>::type;
@@ -408,8 +409,7 @@ void launch_push(const PushArgs<P> &a, int64_t n_bound, cudaStream_t s) {
     } else {
         if (n_bound <= 0) return;
         int64_t blocks = (n_bound + 255) / 256;
-        k_push<P><<<(unsigned)blocks, 256, 0, s>>>(a);
-        PIC_LAUNCHED();
+        launch_chained(a.chain, k_push<P>, (unsigned)blocks, 256, 0, s, a);
     }
 }
 

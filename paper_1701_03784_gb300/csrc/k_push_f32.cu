@@ -265,7 +265,9 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
                                               long long &a1, int &dq0, int &dq1, int4 &EG,
                                               bool &crossed, QEntry &e) {
     const float4 *R = rec4(a.rec, t0);
-    const float4 G = __ldg(R + 0), RH = __ldg(R + 1), CA = __ldg(R + 2), CB = __ldg(R + 3);
+    // the field coefficients are the face kernel's of this step: ordinary loads (the
+    // read-only path is for what no kernel of the chain writes)
+    const float4 G = __ldg(R + 0), RH = __ldg(R + 1), CA = R[2], CB = R[3];
     EG = __ldg(rec4i(a.rec, t0) + 5);   // edges and orientation flags
     const int s2 = LAM_ONE - s0 - s1;
     const float f0 = fix2f(s0), f1 = fix2f(s1), f2 = fix2f(s2);
@@ -462,18 +464,11 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
 }  // namespace
 
 template <bool VAY>
-__global__ void __launch_bounds__(NT, 4) k_push_f32(PushArgs<PF32> a) {
+__global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ PushArgs<PF32> a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     PushSmem &sm = *reinterpret_cast<PushSmem *>(smem_raw);
-    const long long n = *a.n_slots;
-    const long long ntiles = (n + TILE - 1) / TILE;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned full = 0xffffffffu;
-    // each CTA takes a contiguous range of tiles: consecutive tiles hold neighbouring
-    // triangles (slots are sorted by triangle), so their records stay in this SM's L1
-    const long long per = (ntiles + gridDim.x - 1) / gridDim.x;
-    const long long tile0 = (long long)blockIdx.x * per, tile1 = min(ntiles, tile0 + per);
-    if (tile0 >= tile1) return;
     if (tid == 0) {
         for (int s = 0; s < STAGES; s++) {
             mbar_init(&sm.full[s], 1);
@@ -482,6 +477,14 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(PushArgs<PF32> a) {
         mbar_fence_init();
     }
     __syncthreads();
+    chain_wait();
+    const long long n = *a.n_slots;
+    const long long ntiles = (n + TILE - 1) / TILE;
+    // each CTA takes a contiguous range of tiles: consecutive tiles hold neighbouring
+    // triangles (slots are sorted by triangle), so their records stay in this SM's L1
+    const long long per = (ntiles + gridDim.x - 1) / gridDim.x;
+    const long long tile0 = (long long)blockIdx.x * per, tile1 = min(ntiles, tile0 + per);
+    if (tile0 >= tile1) return;
     unsigned cx = 0;
 
     if (warp == CW) {
@@ -598,8 +601,7 @@ static void launch_push_f32_as(const PushArgs<PF32> &a, int64_t n_bound, cudaStr
     const int64_t tiles = (n_bound + TILE - 1) / TILE;
     const int bps = a.ctas_per_sm > 0 ? std::min(a.ctas_per_sm, ps.bps) : ps.bps;
     const int64_t grid = std::min<int64_t>(tiles, (int64_t)ps.sms * bps);
-    k_push_f32<VAY><<<(unsigned)grid, NT, smem, s>>>(a);
-    PIC_LAUNCHED();
+    launch_chained(a.chain, k_push_f32<VAY>, (unsigned)grid, NT, smem, s, a);
 }
 
 void launch_push_f32(const PushArgs<PF32> &a, int64_t n_bound, cudaStream_t s) {

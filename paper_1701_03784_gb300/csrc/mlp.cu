@@ -91,8 +91,7 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 __global__ void k_gather(const float *X, const float *T, float *Xb, float *Tb, long long n, int rows,
                          int mrows, int din, int dout, unsigned long long seed, long long step,
                          int random) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int z = blockIdx.y, w = din + dout;
     const int r = (int)(i / w), k = (int)(i % w);
@@ -305,7 +304,7 @@ struct MlpImpl {
         j.lda = j.kind == MLP_DW ? g.sAk : g.sAm;
         j.ldb = j.kind == MLP_FWD ? g.sBn : g.sBk;
         j.ldc = g.ldc;
-        mlp_jobs(jobs, E, s);
+        mlp_jobs(jobs, E, false, s);
     }
 
     // ---- the FP32 path: every product with what follows it (k_mlp_f32.cu) ----
@@ -336,7 +335,7 @@ struct MlpImpl {
             MlpJobs jobs;
             jobs.job[jobs.n++] = forward_job(l, rows, A, sA, last ? Y + c0 * sz[L] : act[l + 1],
                                              last ? n * sz[L] : (long long)max_batch * sz[l + 1]);
-            mlp_jobs(jobs, E, s);
+            mlp_jobs(jobs, E, l > 0 || c0 > 0, s);
             A = act[l + 1];
             sA = (long long)max_batch * sz[l + 1];
         }
@@ -362,7 +361,7 @@ struct MlpImpl {
                 j.Z = pre[l];
                 j.sZ = sa(l + 1);
             }
-            mlp_jobs(jobs, E, s);
+            mlp_jobs(jobs, E, true, s);
         }
         const auto dx = [&](int l) {
             MlpJob j{};
@@ -411,17 +410,17 @@ struct MlpImpl {
             MlpJobs jobs;
             jobs.job[jobs.n++] = dx(l);
             if (l + 1 < L) jobs.job[jobs.n++] = dw(l + 1);
-            mlp_jobs(jobs, E, s);
+            mlp_jobs(jobs, E, true, s);
         }
         MlpJobs jobs;
         if (L > 1) jobs.job[jobs.n++] = dw(1);
         jobs.job[jobs.n++] = dw(0);
-        mlp_jobs(jobs, E, s);
+        mlp_jobs(jobs, E, true, s);
     }
 
     void gather(int rows, const float *X, const float *T, long long n, unsigned long long seed,
-                long long step, int random, cudaStream_t s) {
-        launch_chained(k_gather, dim3(blocks((long long)rows * (sz[0] + sz[L])), E), 256, 0, s, X, T, act[0],
+                long long step, int random, bool chain, cudaStream_t s) {
+        launch_chained(chain, k_gather, dim3(blocks((long long)rows * (sz[0] + sz[L])), E), 256, 0, s, X, T, act[0],
                        Tb, n, rows, max_batch, sz[0], sz[L], seed, step, random);
     }
     // FP32 inference on n rows by the whole-network kernel, or layer by layer in batches of
@@ -599,7 +598,7 @@ extern "C" pic_status pic_mlp_grad(pic_mlp *m, const float *X, const float *T, i
     }
     cudaStream_t s = (cudaStream_t)st;
     const int rows = (int)n;
-    x.gather(rows, X, T, n, 0, 0, 0, s);
+    x.gather(rows, X, T, n, 0, 0, 0, false, s);
     PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
     if (x.train_tc) {
         x.forward(rows, x.act[0], (long long)x.max_batch * x.sz[0], s);
@@ -635,7 +634,7 @@ extern "C" pic_status pic_mlp_train(pic_mlp *m, const float *X, const float *T, 
     const long long np = x.E * x.P;
     x.touched();
     for (long long k = 0; k < steps; k++) {
-        x.gather(batch, X, T, n, seed, x.adam_step, 1, s);
+        x.gather(batch, X, T, n, seed, x.adam_step, 1, k > 0, s);
         const bool last = k == steps - 1;
         if (last) PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
         x.adam_step++;

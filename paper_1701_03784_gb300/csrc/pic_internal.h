@@ -122,7 +122,7 @@ struct MlpJobs {
     int n = 0;
 };
 // the jobs in one launch (their results must not depend on each other)
-void mlp_jobs(MlpJobs &jobs, int E, cudaStream_t s);
+void mlp_jobs(MlpJobs &jobs, int E, bool chain, cudaStream_t s);
 
 // Parameters as the whole-network kernel reads them: per member and layer the weights
 // k-major (kp x np: kp the inputs up to a multiple of 16, np by mlp_f32_shape) and np biases.
@@ -250,9 +250,17 @@ long long launches_this_thread();
 // statement) until that one has completed and its writes are visible.  The kernel lets its
 // own successor in the same way right after its wait (griddepcontrol.launch_dependents),
 // so that whatever a kernel has waited for has completed before its successor starts.
+// chain = false: an ordinary launch, for the first kernel of a call and for one that
+// follows an event wait (what it depends on is then not a kernel of this stream).
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 template <class... Params, class... Args>
-void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                    Args &&...args) {
+void launch_chained(bool chain, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                    cudaStream_t s, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -262,7 +270,7 @@ void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t sme
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chain ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
     PIC_LAUNCHED();
 }
@@ -323,7 +331,8 @@ enum {
     CNT_EMITTED = 5,    // particles born by the emitter
     CNT_NEXT_PID = 6,   // next particle id once an emitter was set
     CNT_EMIT_DROPPED = 7,   // particles the emitter did not make for lack of room
-    CNT_N = 8
+    CNT_EMIT_TICKET = 8,    // emission blocks done in this step
+    CNT_N = 9
 };
 // slots past the capacity that the particle arrays keep for 16-byte bulk-copy rounding
 constexpr int64_t SLOT_PAD = 8;
@@ -345,6 +354,7 @@ struct PushArgs {
     int32_t ctas_per_sm;        // launch shape: persistent CTAs per SM (0: as many as fit)
     int32_t pusher;             // PIC_PUSHER_BORIS or PIC_PUSHER_VAY (Eq. DLE)
     int64_t wait_polls;         // FP32 kernel: polls before a tile-pipeline wait gives up
+    bool chain = true;          // launched behind a kernel of the step (launch_chained)
 };
 // default of PushArgs::wait_polls (each poll suspends the thread for at most 100 us)
 constexpr int64_t PUSH_WAIT_POLLS = 1LL << 14;
@@ -372,9 +382,6 @@ struct EmitArgs {
     unsigned long long seed;
 };
 
-template <class P>
-void launch_emit(const EmitArgs<P> &a, cudaStream_t s);
-
 // field probes: group g owns entries [ptr[g], ptr[g+1]) of (face, weight); state[0] is
 // the step phase, state[1] the records written, state[2] the records dropped
 template <class P>
@@ -387,15 +394,12 @@ struct ProbeArgs {
     double *buf;            // capacity x n_groups
     long long *state;
     unsigned *done;
-    int32_t n_groups, every;
-    long long capacity;
+    int32_t n_groups = 0, every = 1;
+    long long capacity = 0;
 };
 
-template <class P>
-void launch_probe(const ProbeArgs<P> &a, cudaStream_t s);
-
 // output ports: port k owns entries [ptr[k], ptr[k+1]) of (triangle, barycentric point,
-// quadrature weight); after the face kernel of a step, P_k = sum w E_rho(lambda) B_phi
+// quadrature weight); between the face kernels of two steps, P_k = sum w E_rho(lambda) B_phi
 // from the triangle records (E^n and the time-centred B_phi); every `every` steps the
 // ports' values are appended to a device buffer; state as for the probes
 template <class P>
@@ -408,12 +412,9 @@ struct PortArgs {
     double *buf;            // capacity x n_ports
     long long *state;
     unsigned *done;
-    int32_t n_ports, every;
-    long long capacity;
+    int32_t n_ports = 0, every = 1;
+    long long capacity = 0;
 };
-
-template <class P>
-void launch_port(const PortArgs<P> &a, cudaStream_t s);
 
 template <class P>
 struct FieldArgs {
@@ -449,12 +450,18 @@ struct FieldArgs {
     unsigned long long *counters;
     int64_t N0;
     int32_t block;              // launch shape: threads per block (<= 512)
+    bool chain = true;          // the face kernel is launched behind a kernel of the last step
 };
 
 template <class P> void launch_push(const PushArgs<P> &a, int64_t n_bound, cudaStream_t s);
 void launch_push_f32(const PushArgs<PF32> &a, int64_t n_bound, cudaStream_t s);
-template <class P> void launch_field_b(const FieldArgs<P> &a, cudaStream_t s);
-template <class P> void launch_field_e(const FieldArgs<P> &a, cudaStream_t s);
+// emit: births to make beside the face kernel, or null
+template <class P>
+void launch_field_b(const FieldArgs<P> &a, const EmitArgs<P> *emit, cudaStream_t s);
+// probe, port: recorded beside the residual kernel; no groups, no ports: none
+template <class P>
+void launch_field_e(const FieldArgs<P> &a, const ProbeArgs<P> &probe, const PortArgs<P> &port,
+                    cudaStream_t s);
 template <class P>
 void launch_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, int64_t first,
                       int64_t count, typename P::Acc *Q, cudaStream_t s);

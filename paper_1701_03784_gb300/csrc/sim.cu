@@ -1006,7 +1006,7 @@ struct SimImpl final : SimBase {
     }
 
     // the part of a step before the particle kernel: the Gauss-law reference of a new
-    // state, emission, the face kernel (B update, J / Q_abs cleared), probes and ports
+    // state, the face kernel (B update, J / Q_abs cleared) and emission beside it
     pic_status step_begin(FieldArgs<P> &fa, cudaStream_t s) {
         if (dgl_dirty) {
             // DGL reference res = D_div D^n - Q^n before the first step of this state
@@ -1015,8 +1015,8 @@ struct SimImpl final : SimBase {
                            parts[cur], d_n, n_bound, q_scale(), 0.0, diag_out, s);
             dgl_dirty = false;
         }
+        EmitArgs<P> ea;
         if (emitting) {
-            EmitArgs<P> ea;
             ea.line = eline;
             ea.p = parts[cur];
             ea.rec = rec;
@@ -1031,15 +1031,12 @@ struct SimImpl final : SimBase {
             ea.u_normal = em.u_normal;
             ea.u_thermal = em.u_thermal;
             ea.seed = (unsigned long long)em.seed;
-            launch_emit<P>(ea, s);
         }
         // the face kernel clears J, Q_abs and (FP64) Q^{n+1}; in the FP32 build Q^{n+1} is
         // written whole by the per-node update
         fa.Qn = Qn();
         fa.Qnext = Qbuf[1 - qcur];
-        launch_field_b<P>(fa, s);
-        if (probes_on) launch_probe<P>(probe, s);
-        if (ports_on) launch_port<P>(port, s);
+        launch_field_b<P>(fa, emitting ? &ea : nullptr, s);
         return PIC_OK;
     }
 
@@ -1066,9 +1063,9 @@ struct SimImpl final : SimBase {
     }
 
     // the part of a step after the particle kernel: the E update (edge residual, SpMV,
-    // node charge), the step count and, when due, the re-sort
+    // node charge; probes and ports beside it), the step count and, when due, the re-sort
     void step_end(FieldArgs<P> &fa, cudaStream_t s) {
-        launch_field_e<P>(fa, s);
+        launch_field_e<P>(fa, probes_on ? probe : ProbeArgs<P>{}, ports_on ? port : PortArgs<P>{}, s);
         qcur = 1 - qcur;
         n_steps++;
         if (sort_interval > 0 && ++since_sort >= sort_interval) resort(s);
@@ -1078,6 +1075,7 @@ struct SimImpl final : SimBase {
         stepped = true;
         FieldArgs<P> fa = field_args();
         for (int64_t it = 0; it < n; it++) {
+            fa.chain = it > 0;
             pic_status st = step_begin(fa, s);
             if (st != PIC_OK) return st;
             const PushArgs<P> pa = push_args(parts[cur], d_n);
@@ -1371,6 +1369,7 @@ struct SimImpl final : SimBase {
         pic_status st;
         stepped = true;
         FieldArgs<P> fa = field_args();
+        fa.chain = false;
         if ((st = step_begin(fa, s)) != PIC_OK) return st;
         k_chunk_counts<<<1, 32, 0, s>>>(d_n, d_chunk_n, chunk, RT_CHUNKS);
         PIC_LAUNCHED();
@@ -1390,7 +1389,9 @@ struct SimImpl final : SimBase {
                 v.up += c0;
                 v.uz += c0;
                 v.pid += c0;
-                launch_push<P>(push_args(v, d_chunk_n + c), c1 - c0, s);
+                PushArgs<P> pa = push_args(v, d_chunk_n + c);
+                pa.chain = false;   // it follows the upload's event
+                launch_push<P>(pa, c1 - c0, s);
             }
             if (!resort_due) {
                 PIC_CUDA_TRY(cudaEventRecord(rt_pushc[c], s));
