@@ -201,19 +201,27 @@ void launch_export(Particles<P> p, int64_t n, const TriRec<typename P::R> *, dou
     PIC_LAUNCHED();
 }
 
-template <class Acc>
-__global__ void k_acc_to_double(const Acc *a, double *out, int64_t n, double scale) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if constexpr (std::is_same<Acc, double>::value) out[i] = a[i] * scale;
-    else out[i] = (double)(long long)a[i] * scale;
+// FP64 copies of arrays for a read-back, one launch for all of them (blockIdx.y: which)
+template <class P>
+__global__ void k_read(const __grid_constant__ ReadArgs<P> a, double *out) {
+    const int q = blockIdx.y;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n[q];
+         i += (int64_t)gridDim.x * blockDim.x) {
+        double v;
+        if (a.field[q]) v = (double)a.field[q][i];
+        else if constexpr (P::fixed) v = (double)(long long)a.acc[q][i] * a.scale[q];
+        else v = a.acc[q][i] * a.scale[q];
+        out[a.at[q] + i] = v;
+    }
 }
 
 template <class P>
-void launch_acc_to_double(const typename P::Acc *a, double *out, int64_t n, double scale,
-                          cudaStream_t s) {
-    if (n <= 0) return;
-    k_acc_to_double<typename P::Acc><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, out, n, scale);
+void launch_read(const ReadArgs<P> &a, double *out, cudaStream_t s) {
+    int64_t most = 0;
+    for (int q = 0; q < a.count; q++) most = std::max(most, a.n[q]);
+    if (most <= 0) return;
+    const int64_t blocks = std::min<int64_t>((most + 255) / 256, 608);
+    k_read<P><<<dim3((unsigned)blocks, (unsigned)a.count), 256, 0, s>>>(a, out);
     PIC_LAUNCHED();
 }
 
@@ -227,8 +235,7 @@ void launch_acc_to_double(const typename P::Acc *a, double *out, int64_t n, doub
                                  cudaStream_t);                                                \
     template void launch_export<P>(Particles<P>, int64_t, const TriRec<P::R> *, double *,      \
                                    double *, int64_t *, cudaStream_t);                         \
-    template void launch_acc_to_double<P>(const P::Acc *, double *, int64_t, double,           \
-                                          cudaStream_t);
+    template void launch_read<P>(const ReadArgs<P> &, double *, cudaStream_t);
 PIC_INST(PF32)
 PIC_INST(PF64)
 

@@ -321,15 +321,15 @@ void launch_push(const PushArgs<P> &a, int64_t n_bound, cudaStream_t s) {
 }
 
 // Eq. charge of the particles in slots [first, first + count) (new particles at
-// injection; all of them for the diagnostics).  FP32 build: the fixed-point coordinates of
+// injection; all of them, as far as *n_slots goes, for the diagnostics).  FP32 build: the fixed-point coordinates of
 // the lanes that share a triangle are summed first (sorted slots: most lanes of a warp do),
 // one set of atomics per triangle; sums of at most 32 coordinates < 2^23 fit in 32 bits.
 template <class P>
 __global__ void k_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, int64_t first,
-                            int64_t count, typename P::Acc *Q) {
+                            int64_t count, const int64_t *n_slots, typename P::Acc *Q) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t i = first + k;
-    const int t = k < count ? p.tri[i] : -1;
+    const int t = k < count && (!n_slots || i < *n_slots) ? p.tri[i] : -1;
     if constexpr (P::fixed) {
         const unsigned grp = __match_any_sync(0xffffffffu, t);
         if (t < 0) return;
@@ -352,17 +352,17 @@ __global__ void k_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, in
 
 template <class P>
 void launch_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, int64_t first,
-                      int64_t count, typename P::Acc *Q, cudaStream_t s) {
+                      int64_t count, const int64_t *n_slots, typename P::Acc *Q, cudaStream_t s) {
     if (count <= 0) return;
-    k_deposit_q<P><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(rec, p, first, count, Q);
+    k_deposit_q<P><<<(unsigned)((count + 255) / 256), 256, 0, s>>>(rec, p, first, count, n_slots, Q);
     PIC_LAUNCHED();
 }
 
 template void launch_push<PF32>(const PushArgs<PF32> &, int64_t, cudaStream_t);
 template void launch_push<PF64>(const PushArgs<PF64> &, int64_t, cudaStream_t);
 template void launch_deposit_q<PF32>(const TriRec<float> *, Particles<PF32>, int64_t, int64_t,
-                                     unsigned long long *, cudaStream_t);
+                                     const int64_t *, unsigned long long *, cudaStream_t);
 template void launch_deposit_q<PF64>(const TriRec<double> *, Particles<PF64>, int64_t, int64_t,
-                                     double *, cudaStream_t);
+                                     const int64_t *, double *, cudaStream_t);
 
 }  // namespace pic

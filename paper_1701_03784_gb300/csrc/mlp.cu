@@ -120,6 +120,19 @@ __global__ void k_params_in(const double *src, float *dst, MlpOffsets from, MlpO
     }
 }
 
+// and the way back
+__global__ void k_params_out(const float *src, double *dst, MlpOffsets from, MlpOffsets to, MlpOffsets len,
+                             int L, long long P, long long cP) {
+    const int z = blockIdx.y / L, l = blockIdx.y % L;
+    const float *s = src + z * P;
+    double *d = dst + z * cP;
+    for (long long i = blockIdx.x * blockDim.x + threadIdx.x; i < len.w[l] + len.b[l];
+         i += (long long)gridDim.x * blockDim.x) {
+        if (i < len.w[l]) d[to.w[l] + i] = s[from.w[l] + i];
+        else d[to.b[l] + i - len.w[l]] = s[from.b[l] + i - len.w[l]];
+    }
+}
+
 inline unsigned blocks(long long n, int b = 256) { return (unsigned)((n + b - 1) / b); }
 }  // namespace
 
@@ -435,13 +448,14 @@ struct MlpImpl {
     }
     // parameters changed: the packed copies are out of date
     void touched() { tc_dirty = f32_dirty = true; }
-    // E x cP doubles from E x P floats
-    void unpad(const float *h, double *out) const {
-        for (int z = 0; z < E; z++)
-            for (int l = 0; l < L; l++) {
-                for (long long i = 0; i < len.w[l]; i++) out[z * cP + coff.w[l] + i] = h[z * P + off.w[l] + i];
-                for (long long i = 0; i < len.b[l]; i++) out[z * cP + coff.b[l] + i] = h[z * P + off.b[l] + i];
-            }
+    // E x P floats (parameters or gradients) as E x cP doubles into a host array: converted
+    // on the device (as a vector converted on the host, 1.1M parameters took 1151 us)
+    pic_status to_host(const float *src, double *out, cudaStream_t s) {
+        k_params_out<<<dim3(64, E * L), 256, 0, s>>>(src, stage, off, coff, len, L, P, cP);
+        PIC_LAUNCHED();
+        PIC_CUDA_TRY(cudaMemcpyAsync(out, stage, sizeof(double) * E * cP, cudaMemcpyDeviceToHost, s));
+        PIC_CUDA_TRY(cudaStreamSynchronize(s));
+        return PIC_OK;
     }
 
     // ---- the tensor-core training path: products, then elementwise kernels ----
@@ -580,11 +594,8 @@ extern "C" pic_status pic_mlp_params_get(pic_mlp *m, double *params) try {
         set_error("pic_mlp_params_get: null output");
         return PIC_ERR_ARG;
     }
-    std::vector<float> h(x.E * x.P);
     PIC_CUDA_TRY(cudaDeviceSynchronize());
-    PIC_CUDA_TRY(cudaMemcpy(h.data(), x.params, sizeof(float) * h.size(), cudaMemcpyDeviceToHost));
-    x.unpad(h.data(), params);
-    return PIC_OK;
+    return x.to_host(x.params, params, nullptr);
 }
 PIC_CATCH("pic_mlp_params_get")
 
@@ -609,12 +620,9 @@ extern "C" pic_status pic_mlp_grad(pic_mlp *m, const float *X, const float *T, i
     PIC_CUDA_TRY(cudaGetLastError());
     pic_status ts = x.tc_errors("pic_mlp_grad", s);
     if (ts != PIC_OK) return ts;
-    std::vector<float> h(x.E * x.P), hl(x.E);
-    PIC_CUDA_TRY(cudaMemcpyAsync(h.data(), x.grads, sizeof(float) * h.size(),
-                                 cudaMemcpyDeviceToHost, s));
+    std::vector<float> hl(x.E);
     PIC_CUDA_TRY(cudaMemcpyAsync(hl.data(), x.loss, sizeof(float) * x.E, cudaMemcpyDeviceToHost, s));
-    PIC_CUDA_TRY(cudaStreamSynchronize(s));
-    x.unpad(h.data(), grads);
+    if ((ts = x.to_host(x.grads, grads, s)) != PIC_OK) return ts;
     if (loss)
         for (int z = 0; z < x.E; z++) loss[z] = hl[z];
     return PIC_OK;

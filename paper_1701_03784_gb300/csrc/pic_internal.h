@@ -464,7 +464,7 @@ void launch_field_e(const FieldArgs<P> &a, const ProbeArgs<P> &probe, const Port
                     cudaStream_t s);
 template <class P>
 void launch_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, int64_t first,
-                      int64_t count, typename P::Acc *Q, cudaStream_t s);
+                      int64_t count, const int64_t *n_slots, typename P::Acc *Q, cudaStream_t s);
 
 struct SortScratch {
     int32_t *cnt = nullptr;      // N2 + 1: counts, then write cursors
@@ -502,9 +502,28 @@ void launch_diag(const DiagDev &d, const typename P::Acc *J, const typename P::A
 template <class P>
 void launch_export(Particles<P> p, int64_t n, const TriRec<typename P::R> *rec,
                    double *lam3, double *u3, int64_t *pid, cudaStream_t s);
+// arrays to be read back as FP64: fields as they are, accumulators times a scale; array q's
+// n[q] values go to out + at[q]
 template <class P>
-void launch_acc_to_double(const typename P::Acc *a, double *out, int64_t n, double scale,
-                          cudaStream_t s);
+struct ReadArgs {
+    const typename P::R *field[4] = {};
+    const typename P::Acc *acc[4] = {};
+    double scale[4] = {};
+    int64_t n[4] = {}, at[4] = {};
+    int count = 0;
+    int64_t total = 0;
+    int64_t add(const typename P::R *f, const typename P::Acc *x, double sc, int64_t m) {
+        field[count] = f;
+        acc[count] = x;
+        scale[count] = sc;
+        n[count] = m;
+        at[count] = total;
+        total += m;
+        return at[count++];
+    }
+};
+template <class P>
+void launch_read(const ReadArgs<P> &a, double *out, cudaStream_t s);
 
 }  // namespace pic
 

@@ -461,9 +461,9 @@ def pic_diagnostics(sim, fields=False, stream=None):
     info = pic_mesh_info(sim.mesh)
     E = B = J = None
     if fields:
-        E = np.zeros(info["n_edges"])
-        B = np.zeros(info["n_tris"])
-        J = np.zeros(info["n_edges"])
+        E = np.empty(info["n_edges"])
+        B = np.empty(info["n_tris"])
+        J = np.empty(info["n_edges"])
     _check(_lib.pic_diagnostics(sim.ptr, ctypes.byref(d), _ptr(E), _ptr(B), _ptr(J),
                                 _stream(stream)), "pic_diagnostics")
     out = {k: getattr(d, k) for k, _ in pic_diag._fields_}
@@ -475,8 +475,8 @@ def pic_diagnostics(sim, fields=False, stream=None):
 def pic_fields_get(sim, stream=None):
     """(E on edges, B on faces) as float64 arrays: pic_diagnostics without its reductions."""
     info = pic_mesh_info(sim.mesh)
-    E = np.zeros(info["n_edges"])
-    B = np.zeros(info["n_tris"])
+    E = np.empty(info["n_edges"])
+    B = np.empty(info["n_tris"])
     _check(_lib.pic_diagnostics(sim.ptr, None, _ptr(E), _ptr(B), None, _stream(stream)),
            "pic_diagnostics")
     return E, B
@@ -508,7 +508,7 @@ def pic_charges_get_static(sim, Q=None, Q_prev=None, Q_absorbed=None, stream=Non
 
 def pic_charges_get(sim, stream=None):
     n0 = pic_mesh_info(sim.mesh)["n_nodes"]
-    Q, Qp, Qa = np.zeros(n0), np.zeros(n0), np.zeros(n0)
+    Q, Qp, Qa = np.empty(n0), np.empty(n0), np.empty(n0)
     _check(_lib.pic_charges_get(sim.ptr, _ptr(Q), _ptr(Qp), _ptr(Qa), _stream(stream)),
            "pic_charges_get")
     return Q, Qp, Qa
@@ -523,10 +523,10 @@ def pic_particles_count(sim, stream=None):
 
 def pic_particles_get(sim, stream=None):
     n = pic_particles_count(sim, stream)
-    pid = np.zeros(n, np.int64)
-    tri = np.zeros(n, np.int32)
-    lam = np.zeros((n, 3))
-    u = np.zeros((n, 3))
+    pid = np.empty(n, np.int64)
+    tri = np.empty(n, np.int32)
+    lam = np.empty((n, 3))
+    u = np.empty((n, 3))
     _check(_lib.pic_particles_get(sim.ptr, n, _ptr(pid), _ptr(tri), _ptr(lam), _ptr(u),
                                   _stream(stream)), "pic_particles_get")
     return dict(pid=pid, tri=tri, lam=lam, u=u)
@@ -639,7 +639,7 @@ def pic_mlp_params_set(m, params):
 
 
 def pic_mlp_params_get(m):
-    p = np.zeros((m.members, pic_mlp_param_count(m)))
+    p = np.empty((m.members, pic_mlp_param_count(m)))
     _check(_lib.pic_mlp_params_get(m.ptr, _ptr(p)), "pic_mlp_params_get")
     return p
 
@@ -655,7 +655,7 @@ def pic_mlp_train(m, X, T, batch, steps, lr=1e-3, seed=0, stream=None):
 
 
 def pic_mlp_grad(m, X, T, stream=None):
-    g = np.zeros((m.members, pic_mlp_param_count(m)))
+    g = np.empty((m.members, pic_mlp_param_count(m)))
     loss = np.zeros(m.members)
     _check(_lib.pic_mlp_grad(m.ptr, _dev(X, "X"), _dev(T, "T"), X.shape[0], _ptr(g), _ptr(loss),
                              _stream(stream)), "pic_mlp_grad")
