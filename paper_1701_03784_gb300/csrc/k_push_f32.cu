@@ -60,6 +60,21 @@ __device__ __forceinline__ int f2fix(float x) {
     return __float_as_int(fmaf(x, ONEF, TWO23)) - TWO23_BITS;
 }
 
+// Reciprocal and reciprocal square root of numbers in the normal range: the hardware's
+// approximations alone.  (__fdividef and rsqrtf wrap them in scaling for denormals, whose
+// instructions this kernel, bound by its issue rate, would pay in every push and segment;
+// in the normal range the values are the same.)
+__device__ __forceinline__ float rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rsq(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 __device__ __forceinline__ const float4 *rec4(const TriRec<float> *rec, int t) {
     return reinterpret_cast<const float4 *>(rec + t);
 }
@@ -101,17 +116,22 @@ struct Seg {
     float sx;        // fraction of the remaining displacement used
 };
 
-// End of the segment that starts at f (float of the fixed-point start) and moves by dl,
-// in one triangle.  The exit edge is the one reached first (smallest parameter, ties to
-// the lower index), never the edge just entered; the crossing point has coordinate kx
-// exactly 0 and the other two summing to 2^22.
+// the point of an edge whose two end nodes have coordinates ci, cj (up to a common
+// factor): the first node's share in fixed point
+__device__ __forceinline__ int edge_point(float ci, float cj) {
+    const int q = f2fix(fminf(ci * rcp(ci + cj), 1.f));
+    return min(max(q, 0), LAM_ONE);
+}
+
+// End of a particle's first segment, which starts at f (float of the fixed-point start) and
+// moves by dl, in one triangle.  The exit edge is the one reached first (smallest
+// parameter, ties to the lower index); the crossing point has coordinate kx exactly 0 and
+// the other two summing to 2^22.
 __device__ __forceinline__ Seg segment_end(float f0, float f1, float f2, float dl0, float dl1,
-                                           float dl2, int entered) {
+                                           float dl2) {
     Seg r;
     const float le0 = f0 + dl0, le1 = f1 + dl1, le2 = f2 + dl2;
-    const bool x0 = le0 < 0.f && entered != 0;
-    const bool x1 = le1 < 0.f && entered != 1;
-    const bool x2 = le2 < 0.f && entered != 2;
+    const bool x0 = le0 < 0.f, x1 = le1 < 0.f, x2 = le2 < 0.f;
     if (!(x0 || x1 || x2)) {
         r.kx = -1;
         r.sx = 1.f;
@@ -124,18 +144,16 @@ __device__ __forceinline__ Seg segment_end(float f0, float f1, float f2, float d
         }
         return r;
     }
-    const float sA = x0 ? __fdividef(f0, f0 - le0) : 2.f;
-    const float sB = x1 ? __fdividef(f1, f1 - le1) : 2.f;
-    const float sC = x2 ? __fdividef(f2, f2 - le2) : 2.f;
+    const float sA = x0 ? f0 * rcp(f0 - le0) : 2.f;
+    const float sB = x1 ? f1 * rcp(f1 - le1) : 2.f;
+    const float sC = x2 ? f2 * rcp(f2 - le2) : 2.f;
     if (sA <= sB && sA <= sC) { r.kx = 0; r.sx = sA; }
     else if (sB <= sC) { r.kx = 1; r.sx = sB; }
     else { r.kx = 2; r.sx = sC; }
     const int kx = r.kx;
     const float ci = fmaxf(__fmaf_rn(r.sx, self3(kx, dl1, dl2, dl0), self3(kx, f1, f2, f0)), 0.f);
     const float cj = fmaxf(__fmaf_rn(r.sx, self3(kx, dl2, dl0, dl1), self3(kx, f2, f0, f1)), 0.f);
-    int qi = f2fix(fminf(__fdividef(ci, ci + cj), 1.f));
-    qi = min(max(qi, 0), LAM_ONE);
-    const int qj = LAM_ONE - qi;
+    const int qi = edge_point(ci, cj), qj = LAM_ONE - qi;
     r.e0 = kx == 0 ? 0 : (kx == 1 ? qj : qi);
     r.e1 = kx == 1 ? 0 : (kx == 2 ? qj : qi);
     r.e2 = kx == 2 ? 0 : (kx == 0 ? qj : qi);
@@ -160,14 +178,6 @@ __device__ __forceinline__ void oriented(int flags, long long &A0, long long &A1
     if (!(flags & 1)) A0 = -A0;
     if (!(flags & 2)) A1 = -A1;
     if (!(flags & 4)) A2 = -A2;
-}
-
-// the three oriented currents of one segment s -> e
-__device__ __forceinline__ void currents(int s0, int s1, int s2, const Seg &e, int flags,
-                                         long long &J0, long long &J1, long long &J2) {
-    J1 = (long long)s2 * e.e0 - (long long)s0 * e.e2;
-    ccw_from(J1, s0 - e.e0, s1 - e.e1, J0, J2);
-    oriented(flags, J0, J1, J2);
 }
 
 // a particle whose displacement leaves its start triangle t: slot, start point (s0, s1,
@@ -283,7 +293,7 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
         // solved in closed form: u' = u + 2h E + h (u / gamma) x B, tau = h B, gamma_new^2
         // the positive root of g^4 - sigma g^2 - (tau^2 + (u'.tau)^2 / c^2),
         // t = tau / gamma_new, u = (u' + (u'.t) t + u' x t) / (1 + t^2)
-        const float gi = rsqrtf(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
+        const float gi = rsq(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
         const float tp = h * CB.z, tz = h * a.bz;
         const float pr = ur + 2.f * h * Er + gi * (up * tz - uz * tp);
         const float pp = up - gi * ur * tz;
@@ -293,11 +303,11 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
         const float x = tau2 + ut0 * ut0 * a.inv_c2;
         const float sigma = 1.f + (pr * pr + pp * pp + pz * pz) * a.inv_c2 - tau2;
         const float disc = sqrtf(sigma * sigma + 4.f * x);
-        const float g2 = sigma >= 0.f ? 0.5f * (sigma + disc) : __fdividef(2.f * x, disc - sigma);
-        const float gn = rsqrtf(g2);
+        const float g2 = sigma >= 0.f ? 0.5f * (sigma + disc) : 2.f * x * rcp(disc - sigma);
+        const float gn = rsq(g2);
         const float qp = tp * gn, qz = tz * gn;
         const float ut = pp * qp + pz * qz;
-        const float sf = __fdividef(1.f, 1.f + qp * qp + qz * qz);
+        const float sf = rcp(1.f + qp * qp + qz * qz);
         ur = sf * (pr + pp * qz - pz * qp);
         up = sf * (pp + ut * qp - pr * qz);
         uz = sf * (pz + ut * qz + pr * qp);
@@ -306,9 +316,9 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
         // kick
         ur += h * Er;
         uz += h * Ez;
-        const float gi = rsqrtf(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
+        const float gi = rsq(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
         const float tp = h * CB.z * gi, tz = h * a.bz * gi;
-        const float sf = __fdividef(2.f, 1.f + tp * tp + tz * tz);
+        const float sf = 2.f * rcp(1.f + tp * tp + tz * tz);
         const float pr = ur + (up * tz - uz * tp);   // u' = u- + u- x t, t = (0, tp, tz)
         const float pp = up - ur * tz;
         const float pz = uz + ur * tp;
@@ -318,15 +328,15 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
     }
 
     // move (Eq. DNE) in the ring's Cartesian frame, rotate back to the meridian plane
-    const float gi = rsqrtf(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
+    const float gi = rsq(1.f + (ur * ur + up * up + uz * uz) * a.inv_c2);
     const float xr = ur * gi * a.dt, yp = up * gi * a.dt;
     const float x = rho + xr;
     const float rn2 = x * x + yp * yp;
     const float d0 = uz * gi * a.dt;
     float d1 = 0.f;
-    if (rn2 > 0.f) {
-        const float rinv = rsqrtf(rn2);
-        d1 = __fdividef(2.f * rho * xr + xr * xr + yp * yp, rn2 * rinv + rho);
+    if (rn2 >= 1.17549435e-38f) {   // normal: on the axis there is no direction to turn
+        const float rinv = rsq(rn2);
+        d1 = (2.f * rho * xr + xr * xr + yp * yp) * rcp(rn2 * rinv + rho);
         const float cs = x * rinv, sn = yp * rinv;
         const float nr = cs * ur + sn * up;
         up = -sn * ur + cs * up;
@@ -393,7 +403,7 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
     if (valid) {
         EG = __ldg(rec4i(a.rec, t) + 5);   // edges, orientation flags
         NB = __ldg(rec4i(a.rec, t) + 6);   // neighbours, entry indices
-        sg = segment_end(fix2f(s0), fix2f(s1), fix2f(s2), q.dl0, q.dl1, -(q.dl0 + q.dl1), -1);
+        sg = segment_end(fix2f(s0), fix2f(s1), fix2f(s2), q.dl0, q.dl1, -(q.dl0 + q.dl1));
         a1 = (long long)s2 * sg.e0 - (long long)s0 * sg.e2;
         dq0 = s0 - sg.e0;
         dq1 = s1 - sg.e1;
@@ -414,37 +424,33 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
             red_add(a.J + EG.z, S2);
         }
     }
-    float d0 = q.d0, d1 = q.d1;
-    for (int ncross = 0;; ncross++) {
-        if (sg.kx < 0) {
-            store_position(a, q.slot, t, sg.e0, sg.e1);
-            return (unsigned)ncross;
-        }
-        const int kx = sg.kx;
+    // From here on a triangle is seen from the edge j that the particle entered by: R is the
+    // coordinate of node j (0 at the start of the segment), P and Q those of nodes j+1 and
+    // j+2, so that only the edges opposite P and Q can be reached, two of the three currents
+    // are single products, and each choice is between two.  The body has no branches but
+    // the loop's exits, and what a finished particle needs is done once after the loop, by
+    // all lanes together.
+    int kx = sg.kx;                                // the edge reached, and its point:
+    int ea = sel3(kx, sg.e1, sg.e2, sg.e0);        // coordinates at nodes kx+1
+    int eb = sel3(kx, sg.e2, sg.e0, sg.e1);        // and kx+2
+    int l0 = sg.e0, l1 = sg.e1;
+    float sx = sg.sx, d0 = q.d0, d1 = q.d1;
+    unsigned ncross = 0;
+    int stop = 0;   // what ended the walk short of the end point: 1 a wall, 2 the walk cap
+    while (kx >= 0) {
+        ncross++;
         const int nb = sel3(kx, NB.x, NB.y, NB.z);
-        if (nb < 0 && -nb == PIC_BC_AXIS) {
-            store_position(a, q.slot, t, sg.e0, sg.e1);
-            return (unsigned)ncross + 1;
-        }
-        if (nb < 0 || ncross + 1 >= a.walk_cap) {
-            const int4 nd = __ldg(rec4i(a.rec, t) + 4);
-            red_add(a.Qabs + nd.x, sg.e0);
-            red_add(a.Qabs + nd.y, sg.e1);
-            red_add(a.Qabs + nd.z, sg.e2);
-            if (nb >= 0) atomicAdd(a.counters + CNT_OVERFLOW, 1ULL);
-            atomicAdd(a.counters + CNT_ABSORBED, 1ULL);
-            __stcs(a.p.tri + q.slot, -1);
-            return (unsigned)ncross + 1;
+        if (nb < 0 || (int)ncross >= a.walk_cap) {
+            l0 = sel3(kx, 0, eb, ea);
+            l1 = sel3(kx, ea, 0, eb);
+            stop = nb >= 0 ? 2 : -nb == PIC_BC_AXIS ? 0 : 1;   // it stays on the axis
+            break;
         }
         // enter nb through its local edge j (opposite its node j): its node j+2 is node kx+1
         // of t, its node j+1 is node kx+2
         const int j = (NB.w >> (2 * kx)) & 3;
-        const int ea = sel3(kx, sg.e1, sg.e2, sg.e0);
-        const int eb = sel3(kx, sg.e2, sg.e0, sg.e1);
-        s0 = j == 0 ? 0 : (j == 1 ? ea : eb);
-        s1 = j == 1 ? 0 : (j == 2 ? ea : eb);
-        s2 = j == 2 ? 0 : (j == 0 ? ea : eb);
-        const float rest = 1.f - sg.sx;
+        const int P = eb, Q = ea;
+        const float rest = 1.f - sx;
         d0 = __fmul_rn(d0, rest);
         d1 = __fmul_rn(d1, rest);
         t = nb;
@@ -452,13 +458,57 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         EG = __ldg(rec4i(a.rec, t) + 5);
         NB = __ldg(rec4i(a.rec, t) + 6);
         const float dl0 = bary_step(G.x, G.y, d0, d1), dl1 = bary_step(G.z, G.w, d0, d1);
-        sg = segment_end(fix2f(s0), fix2f(s1), fix2f(s2), dl0, dl1, -(dl0 + dl1), j);
-        long long J0, J1, J2;
-        currents(s0, s1, s2, sg, EG.w, J0, J1, J2);
-        red_add(a.J + EG.x, J0);
-        red_add(a.J + EG.y, J1);
-        red_add(a.J + EG.z, J2);
+        const float dl2 = -(dl0 + dl1);
+        const float dR = self3(j, dl0, dl1, dl2), dP = self3(j, dl1, dl2, dl0), dQ = self3(j, dl2, dl0, dl1);
+        const float fP = fix2f(P), fQ = fix2f(Q);
+        const float leP = fP + dP, leQ = fQ + dQ;
+        const bool xP = leP < 0.f, xQ = leQ < 0.f, leaves = xP || xQ;
+        // leaving: the edge reached first, opposite P or opposite Q, and the point on it
+        float sP = fP * rcp(fP - leP), sQ = fQ * rcp(fQ - leQ);
+        sP = xP ? sP : 2.f;
+        sQ = xQ ? sQ : 2.f;
+        const bool atP = sP <= sQ;
+        sx = atP ? sP : sQ;
+        const float cR = fmaxf(__fmul_rn(sx, dR), 0.f);
+        const float cS = fmaxf(__fmaf_rn(sx, atP ? dQ : dP, atP ? fQ : fP), 0.f);
+        const int qS = edge_point(cS, cR), qR = LAM_ONE - qS;
+        ea = atP ? qS : qR;
+        eb = atP ? qR : qS;
+        // staying: R takes what rounding leaves, a deficit goes to the larger of P and Q
+        int iP = f2fix(fmaxf(leP, 0.f)), iQ = f2fix(fmaxf(leQ, 0.f));
+        const int iR = LAM_ONE - iP - iQ, neg = min(iR, 0);
+        const bool bigP = iP >= iQ;
+        iP += bigP ? neg : 0;
+        iQ += bigP ? 0 : neg;
+        const int eP = leaves ? (atP ? 0 : qS) : iP;
+        const int eQ = leaves ? (atP ? qS : 0) : iQ;
+        const int eR = leaves ? qR : iR - neg;
+        // Eq. current on edges j (P -> Q), j+1 (Q -> R) and j+2 (R -> P), in their global
+        // orientations
+        const int fl = (EG.w | (EG.w << 3)) >> j;
+        const bool f0 = fl & 1, f1 = fl & 2, f2 = fl & 4;
+        red_add(a.J + sel3(j, EG.x, EG.y, EG.z),
+                (long long)(f0 ? P : -P) * eQ + (long long)(f0 ? -Q : Q) * eP);
+        red_add(a.J + sel3(j, EG.y, EG.z, EG.x), (long long)(f1 ? Q : -Q) * eR);
+        red_add(a.J + sel3(j, EG.z, EG.x, EG.y), (long long)(f2 ? -P : P) * eR);
+        l0 = sel3(j, eR, eQ, eP);
+        l1 = sel3(j, eP, eR, eQ);
+        kx = atP ? (j == 2 ? 0 : j + 1) : (j == 0 ? 2 : j - 1);
+        kx = leaves ? kx : -1;
     }
+    if (stop) {
+        // removed: its charge goes to Q_abs at the point reached
+        const int4 nd = __ldg(rec4i(a.rec, t) + 4);
+        red_add(a.Qabs + nd.x, l0);
+        red_add(a.Qabs + nd.y, l1);
+        red_add(a.Qabs + nd.z, LAM_ONE - l0 - l1);
+        if (stop == 2) atomicAdd(a.counters + CNT_OVERFLOW, 1ULL);
+        atomicAdd(a.counters + CNT_ABSORBED, 1ULL);
+        __stcs(a.p.tri + q.slot, -1);
+    } else {
+        store_position(a, q.slot, t, l0, l1);
+    }
+    return ncross;
 }
 
 }  // namespace
