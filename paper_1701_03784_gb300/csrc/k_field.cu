@@ -25,8 +25,9 @@ __device__ __forceinline__ R along(R e, bool fwd) { return fwd ? e : -e; }
 // it drives the particles but takes no part in the leapfrog), and
 // B_phi = (B^{n+1/2} + B^{n-1/2}) / (2A) (W2 = 1/A).  In a lossy layer
 // B^{n+1/2} = a_f B^{n-1/2} - b_f dt (D_curl E^n)_f.
-// The same launch clears the step's accumulators (J per edge, Q_abs per node, and in the
-// FP64 build Q^{n+1}, which the particle kernel accumulates).  Its first emit_blocks blocks
+// The same launch clears the step's accumulators (the current sums per triangle, in the
+// FP64 build J per edge; Q_abs per node; and in the FP64 build Q^{n+1}, which the particle
+// kernel accumulates).  Its first emit_blocks blocks
 // make the step's births (emit.h).
 // The record is read and written in 16-byte words (g | rho, 1/A | c0 c1 c2, B_phi, pad |
 // nodes, flags | edges, flags); in 8-byte ones the FP64 build's stores alone kept a launch
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
     }
     const int64_t f = (int64_t)(blockIdx.x - (EMIT ? emit_blocks : 0)) * blockDim.x + threadIdx.x;
     const bool face = f < a.N2;
-    R g[2][2] = {}, inv_area = 0;
+    R g[2][2] = {}, inv_area = 0, mu = 0;
     int4 EG = make_int4(0, 0, 0, 0);
     if (face) {
         const R *rc = reinterpret_cast<const R *>(a.rec + f);
@@ -59,9 +60,11 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
         g[1][1] = w[3];
         inv_area = w[7];
         EG = *reinterpret_cast<const int4 *>(a.rec[f].edge);
+        if constexpr (P::fixed) mu = a.mu_inv[f];
     }
     chain_wait();
-    if (f < a.N1) a.J[f] = 0;
+    if constexpr (!P::fixed)
+        if (f < a.N1) a.J[f] = 0;
     if (f < a.N0) {
         a.Qabs[f] = 0;
         if constexpr (!P::fixed) a.Qnext[f] = 0;
@@ -83,6 +86,11 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
     R Bnew = Bold - a.dt * curl;
     if constexpr (LOSS) Bnew = a.loss_f[2 * f] * Bold - a.loss_f[2 * f + 1] * (a.dt * curl);
     a.B[f] = Bnew;
+    if constexpr (P::fixed) {
+        longlong2 *fs = reinterpret_cast<longlong2 *>(a.face + f);
+        fs[0] = make_longlong2(0, 0);
+        fs[1] = make_longlong2(0, __double_as_longlong((double)mu * (double)Bnew));
+    }
     R w[8];
 #pragma unroll
     for (int d = 0; d < 2; d++) {
@@ -98,28 +106,19 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
     for (int k = 0; k < 8; k += W) *reinterpret_cast<R4 *>(out + k) = *reinterpret_cast<R4 *>(w + k);
 }
 
-// Per node, after the particle step.  FP32 build: Q^{n+1} = Q^n - (D_div J)/2^22 -
-// Q_absorbed.  Per particle, the segment currents at a node sum to 2^22 (lambda^start -
-// lambda^end) in the fixed-point units (the identity behind Eq. DCE), so D_div J is
-// divisible by 2^22 and the result equals Eq. charge evaluated at the new positions
-// exactly; a non-zero remainder would be a broken invariant and is counted.  Both builds:
-// the charge removed at walls is summed since the Gauss-law reference.
-template <class P>
-__device__ __forceinline__ void node_update(const FieldArgs<P> &a, int64_t k) {
-    if constexpr (P::fixed) {
-        long long div = 0;
-        for (int64_t q = a.node_ptr[k]; q < a.node_ptr[k + 1]; q++)
-            div += (long long)a.node_sign[q] * (long long)a.J[a.node_edge[q]];
-        if (div & (long long)(LAM_ONE - 1)) atomicAdd(a.counters + CNT_REMAINDER, 1ULL);
-        long long qn = (long long)a.Qn[k] - (div >> LAM_BITS) - (long long)a.Qabs[k];
-        a.Qnext[k] = (unsigned long long)qn;
-    }
-    a.Qwall[k] += a.Qabs[k];
-}
-
-// K4a, one thread per free edge: r = D_curl^T star_mu^-1 B^{n+1/2} - J^{n+1/2}; the DGL
-// auxiliary flux D += dt r.  The same launch does the per-node update (thread k, node k),
-// and its first blocks record probes and ports (record.h).
+// K4a, one thread per edge: in the FP32 build its current from the sums of its triangles;
+// on free edges r = D_curl^T star_mu^-1 B^{n+1/2} - J^{n+1/2} and the DGL auxiliary flux
+// D += dt r.  The first blocks record probes and ports (record.h).
+//
+// One thread per node, in the same launch: in the FP32 build Q^{n+1} = Q^n - (D_div J)/2^22
+// - Q_absorbed, where (D_div J)/2^22 is the charge that left the node through its triangles
+// (FaceSum), which equals Eq. charge evaluated at the new positions exactly (the
+// diagnostics compare); in both builds the charge removed at walls is summed since the
+// Gauss-law reference.
+//
+// Bound by the sectors it gathers from triangles that lie anywhere in memory: two an edge
+// and six a node, of 32 bytes each (with B, star_mu^-1 and the sums in arrays of their own
+// it was six an edge, and eight surrogate instances' 64 steps took 2956 us instead of 2676).
 template <class P, bool REC>
 __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldArgs<P> a,
                                                  const __grid_constant__ ProbeArgs<P> probe,
@@ -135,37 +134,79 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
         }
         blk -= probe.n_groups + port.n_ports;
     }
-    const int64_t i = (int64_t)blk * blockDim.x + threadIdx.x;
-    int32_t e = 0;
-    int2 ef = make_int2(0, 0);
-    if (i < a.nf) {
-        e = a.free_edges[i];
-        ef = reinterpret_cast<const int2 *>(a.edge_face)[i];
-    }
+    const int64_t e = (int64_t)blk * blockDim.x + threadIdx.x;
+    int fs[2] = {0, 0}, i = -1;
     R mu[2] = {0, 0};
+    if (e < a.N1) {
+        const int2 ef = reinterpret_cast<const int2 *>(a.edge_face)[e];
+        fs[0] = ef.x;
+        fs[1] = ef.y;
+        i = a.free_of_edge[e];
+    }
+    // a node's triangles: the first NEAR of them before the wait (six on average)
+    constexpr int NEAR = P::fixed ? 7 : 1;
+    int near[NEAR], q0 = 0, q1 = 0;
+    if constexpr (P::fixed) {
+        if (e < a.N0) {
+            q0 = a.face_ptr[e];
+            q1 = a.face_ptr[e + 1];
+        }
 #pragma unroll
-    for (int q = 0; q < 2; q++) {
-        const int32_t fs = q == 0 ? ef.x : ef.y;
-        if (fs != 0) mu[q] = a.mu_inv[(fs > 0 ? fs : -fs) - 1];
+        for (int q = 0; q < NEAR; q++)
+            if (q0 + q < q1) near[q] = a.node_face[q0 + q];
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+            if (fs[q] != 0) mu[q] = a.mu_inv[(abs(fs[q]) - 1) >> 2];
     }
     chain_wait();
-    if (i < a.N0) node_update<P>(a, i);
-    if (i >= a.nf) return;
-    double r = 0;
+    if (e < a.N1) {
+        double r = 0;
+        long long J = 0;
 #pragma unroll
-    for (int q = 0; q < 2; q++) {
-        int32_t fs = q == 0 ? ef.x : ef.y;
-        if (fs == 0) continue;
-        int32_t f = (fs > 0 ? fs : -fs) - 1;
-        double hf = (double)mu[q] * (double)a.B[f];
-        r += fs > 0 ? hf : -hf;
+        for (int q = 0; q < 2; q++) {
+            if (fs[q] == 0) continue;
+            const int fk = abs(fs[q]) - 1, f = fk >> 2;
+            double hf;
+            if constexpr (P::fixed) {
+                const longlong2 *F = reinterpret_cast<const longlong2 *>(a.face + f);
+                const longlong2 d = F[0], ah = F[1];
+                long long A = ah.x;                                  // edge 1
+                if ((fk & 3) != 1) A += d.x << LAM_BITS;             // edge 2
+                if ((fk & 3) == 0) A += d.y << LAM_BITS;             // edge 0
+                J += fs[q] > 0 ? A : -A;
+                hf = __longlong_as_double(ah.y);
+            } else {
+                hf = mu[q] * a.B[f];
+            }
+            r += fs[q] > 0 ? hf : -hf;
+        }
+        if constexpr (P::fixed) a.J[e] = (unsigned long long)J;
+        if (i >= 0) {
+            double Jp;
+            if constexpr (P::fixed) Jp = (double)J * a.j_scale;
+            else Jp = a.J[e] * a.j_scale;
+            r -= Jp;
+            a.D[e] += (double)a.dt * r;
+            a.r[i] = (R)r;
+        }
     }
-    double Jp;
-    if constexpr (P::fixed) Jp = (double)(long long)a.J[e] * a.j_scale;
-    else Jp = a.J[e] * a.j_scale;
-    r -= Jp;
-    a.D[e] += (double)a.dt * r;
-    a.r[i] = (R)r;
+    if (e >= a.N0) return;
+    const typename P::Acc gone = a.Qabs[e];
+    if constexpr (P::fixed) {
+        long long out = 0;
+        const auto left = [&](int fk) {
+            const longlong2 d = *reinterpret_cast<const longlong2 *>(a.face + (fk >> 2));
+            const int k = fk & 3;
+            out += k == 0 ? d.x : k == 1 ? d.y : -(d.x + d.y);
+        };
+#pragma unroll
+        for (int q = 0; q < NEAR; q++)
+            if (q0 + q < q1) left(near[q]);
+        for (int q = q0 + NEAR; q < q1; q++) left(a.node_face[q]);
+        a.Qnext[e] = a.Qn[e] - (unsigned long long)out - gone;
+    }
+    a.Qwall[e] += gone;
 }
 
 // K4b, sliced ELL SpMV over free edges: E_e += dt (M r)_i (in a lossy layer
@@ -233,7 +274,7 @@ __global__ void __launch_bounds__(512) k_field_spmv(const __grid_constant__ Fiel
 
 template <class P>
 void launch_field_b(const FieldArgs<P> &a, const EmitArgs<P> *emit, cudaStream_t s) {
-    const int64_t n = std::max(a.N2, std::max(a.N1, a.N0));
+    const int64_t n = std::max(a.N2, P::fixed ? a.N0 : std::max(a.N1, a.N0));
     const int b = a.block;
     const bool births = emit && emit->per_step > 0 && emit->line.n > 0;
     const EmitArgs<P> em = births ? *emit : EmitArgs<P>{};
@@ -259,7 +300,7 @@ void launch_field_b(const FieldArgs<P> &a, const EmitArgs<P> *emit, cudaStream_t
 template <class P>
 void launch_field_e(const FieldArgs<P> &a, const ProbeArgs<P> &probe, const PortArgs<P> &port,
                     cudaStream_t s) {
-    const int64_t n = std::max(a.nf, a.N0);
+    const int64_t n = std::max(a.N1, a.N0);
     const int b = a.block, nr = probe.n_groups + port.n_ports;
     const unsigned g = (unsigned)((n + b - 1) / b + nr);
     if (nr > 0) launch_chained(true, k_field_r<P, true>, g, b, 0, s, a, probe, port);

@@ -16,9 +16,11 @@
 //    buffer is refilled once all compute warps have arrived on its "empty" mbarrier;
 //  * 8 compute warps advance two slots per thread per tile, branch-free: gather, push,
 //    rotate-back and the end point in the start triangle.  For the ~4 in 5 particles
-//    whose end point stays there, the edge currents are summed over the lanes that
-//    share the triangle (match.any, then redux.sync on two 23-bit limbs) and one lane
-//    per triangle issues the atomics.  A particle that leaves its triangle is appended,
+//    whose end point stays there, the currents are summed over the lanes that share the
+//    triangle (match.any, then redux.sync on two 23-bit limbs) and one lane per triangle
+//    adds them to the triangle's sums (FaceSum; edge by edge in the global orientations
+//    here, a launch on 16M particles took 283 us and 478 warp instructions per 32 of them
+//    instead of 259 us and 427).  A particle that leaves its triangle is appended,
 //    with its start point and displacement, to its warp's ring in shared memory;
 //  * whenever 32 entries are waiting, the warp walks them with all lanes: per triangle
 //    the segment to the first edge reached, its currents (direct atomics), then the
@@ -160,24 +162,13 @@ __device__ __forceinline__ Seg segment_end(float f0, float f1, float f2, float d
     return r;
 }
 
-// Eq. current of a segment s -> e inside one triangle.  With the local edges oriented
-// counter-clockwise (edge 0: 1->2, 1: 2->0, 2: 0->1) the currents are
-//   A0 = s1 e2 - s2 e1,  A1 = s2 e0 - s0 e2,  A2 = s0 e1 - s1 e0,
-// and because s and e both sum to 2^22, the net outflow at each node is
-//   A2 - A1 = 2^22 (s0 - e0),  A0 - A2 = 2^22 (s1 - e1)   (the identity behind Eq. DCE).
-// So one 64-bit product pair (A1) and two 32-bit differences determine all three, also
-// after summing over particles of the same triangle.
-__device__ __forceinline__ void ccw_from(long long A1, int d0, int d1, long long &A0,
-                                         long long &A2) {
-    A2 = A1 + ((long long)d0 << LAM_BITS);
-    A0 = A2 + ((long long)d1 << LAM_BITS);
-}
-// the ccw currents with the global orientation of each edge applied (flags bit k: local
-// edge k runs (k+1)%3 -> (k+2)%3, i.e. from its lower to its higher node index)
-__device__ __forceinline__ void oriented(int flags, long long &A0, long long &A1, long long &A2) {
-    if (!(flags & 1)) A0 = -A0;
-    if (!(flags & 2)) A1 = -A1;
-    if (!(flags & 4)) A2 = -A2;
+// adds a triangle's current sums of this warp, or of one segment (FaceSum)
+__device__ __forceinline__ void add_current(const PushArgs<PF32> &a, int t, long long a1, long long d0,
+                                            long long d1) {
+    unsigned long long *f = reinterpret_cast<unsigned long long *>(a.face + t);
+    atomicAdd(f, (unsigned long long)d0);
+    atomicAdd(f + 1, (unsigned long long)d1);
+    atomicAdd(f + 2, (unsigned long long)a1);
 }
 
 // a particle whose displacement leaves its start triangle t: slot, start point (s0, s1,
@@ -266,19 +257,18 @@ __device__ __forceinline__ void issue_tile(const PushArgs<PF32> &a, PushSmem &sm
 
 // Gather, push, rotate-back and the end of the move for one particle (slot i, state from
 // the staged tile).  A particle whose end point stays in its start triangle t0 gets its
-// current as (A1, s0 - e0, s1 - e1) (see ccw_from) and its new position stored; one that
+// current as (A1, s0 - e0, s1 - e1) (see FaceSum) and its new position stored; one that
 // leaves t0 is described in e, flagged, and contributes no current here (its whole path,
 // the part in t0 included, is walked later).
 template <bool VAY>
 __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, int t0, int s0,
                                               int s1, float ur, float up, float uz,
-                                              long long &a1, int &dq0, int &dq1, int4 &EG,
-                                              bool &crossed, QEntry &e) {
+                                              long long &a1, int &dq0, int &dq1, bool &crossed,
+                                              QEntry &e) {
     const float4 *R = rec4(a.rec, t0);
     // the field coefficients are the face kernel's of this step: ordinary loads (the
     // read-only path is for what no kernel of the chain writes)
     const float4 G = __ldg(R + 0), RH = __ldg(R + 1), CA = R[2], CB = R[3];
-    EG = __ldg(rec4i(a.rec, t0) + 5);   // edges and orientation flags
     const int s2 = LAM_ONE - s0 - s1;
     const float f0 = fix2f(s0), f1 = fix2f(s1), f2 = fix2f(s2);
 
@@ -396,12 +386,11 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
     const unsigned full = 0xffffffffu;
     int t = valid ? q.t : -1;
     int s0 = q.s0, s1 = q.s1, s2 = LAM_ONE - q.s0 - q.s1;
-    int4 EG = make_int4(0, 0, 0, 0), NB = EG;
+    int4 NB = make_int4(0, 0, 0, 0);
     Seg sg{};
     long long a1 = 0;
     int dq0 = 0, dq1 = 0;
     if (valid) {
-        EG = __ldg(rec4i(a.rec, t) + 5);   // edges, orientation flags
         NB = __ldg(rec4i(a.rec, t) + 6);   // neighbours, entry indices
         sg = segment_end(fix2f(s0), fix2f(s1), fix2f(s2), q.dl0, q.dl1, -(q.dl0 + q.dl1));
         a1 = (long long)s2 * sg.e0 - (long long)s0 * sg.e2;
@@ -415,19 +404,12 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         long long S1 = group_sum(grp, cnt, a1);
         const int D0 = (int)__reduce_add_sync(grp, (unsigned)dq0);
         const int D1 = (int)__reduce_add_sync(grp, (unsigned)dq1);
-        if (lane == __ffs(grp) - 1) {
-            long long S0, S2;
-            ccw_from(S1, D0, D1, S0, S2);
-            oriented(EG.w, S0, S1, S2);
-            red_add(a.J + EG.x, S0);
-            red_add(a.J + EG.y, S1);
-            red_add(a.J + EG.z, S2);
-        }
+        if (lane == __ffs(grp) - 1) add_current(a, t, S1, D0, D1);
     }
     // From here on a triangle is seen from the edge j that the particle entered by: R is the
     // coordinate of node j (0 at the start of the segment), P and Q those of nodes j+1 and
-    // j+2, so that only the edges opposite P and Q can be reached, two of the three currents
-    // are single products, and each choice is between two.  The body has no branches but
+    // j+2, so that only the edges opposite P and Q can be reached and each choice is between
+    // two.  The body has no branches but
     // the loop's exits, and what a finished particle needs is done once after the loop, by
     // all lanes together.
     int kx = sg.kx;                                // the edge reached, and its point:
@@ -455,7 +437,6 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         d1 = __fmul_rn(d1, rest);
         t = nb;
         const float4 G = __ldg(rec4(a.rec, t));
-        EG = __ldg(rec4i(a.rec, t) + 5);
         NB = __ldg(rec4i(a.rec, t) + 6);
         const float dl0 = bary_step(G.x, G.y, d0, d1), dl1 = bary_step(G.z, G.w, d0, d1);
         const float dl2 = -(dl0 + dl1);
@@ -483,16 +464,12 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         const int eP = leaves ? (atP ? 0 : qS) : iP;
         const int eQ = leaves ? (atP ? qS : 0) : iQ;
         const int eR = leaves ? qR : iR - neg;
-        // Eq. current on edges j (P -> Q), j+1 (Q -> R) and j+2 (R -> P), in their global
-        // orientations
-        const int fl = (EG.w | (EG.w << 3)) >> j;
-        const bool f0 = fl & 1, f1 = fl & 2, f2 = fl & 4;
-        red_add(a.J + sel3(j, EG.x, EG.y, EG.z),
-                (long long)(f0 ? P : -P) * eQ + (long long)(f0 ? -Q : Q) * eP);
-        red_add(a.J + sel3(j, EG.y, EG.z, EG.x), (long long)(f1 ? Q : -Q) * eR);
-        red_add(a.J + sel3(j, EG.z, EG.x, EG.y), (long long)(f2 ? -P : P) * eR);
+        // Eq. current from (0, P, Q) at nodes (j, j+1, j+2)
         l0 = sel3(j, eR, eQ, eP);
         l1 = sel3(j, eP, eR, eQ);
+        const int t0 = sel3(j, 0, Q, P), t1 = sel3(j, P, 0, Q);
+        add_current(a, t, (long long)(LAM_ONE - t0 - t1) * l0 - (long long)t0 * (LAM_ONE - l0 - l1), t0 - l0,
+                    t1 - l1);
         kx = atP ? (j == 2 ? 0 : j + 1) : (j == 0 ? 2 : j - 1);
         kx = leaves ? kx : -1;
     }
@@ -582,12 +559,11 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
                 const int t0 = i < n ? b.tri[k] : -1;
                 long long a1 = 0;
                 int dq0 = 0, dq1 = 0;
-                int4 EG = make_int4(0, 0, 0, 0);
                 bool crossed = false;
                 QEntry e;
                 if (t0 >= 0)
                     push_particle<VAY>(a, (int)i, t0, b.l0[k], b.l1[k], b.ur[k], b.up[k], b.uz[k],
-                                       a1, dq0, dq1, EG, crossed, e);
+                                       a1, dq0, dq1, crossed, e);
                 // currents of the particles that stay: summed over the lanes of each start
                 // triangle (one 64-bit and two 32-bit sums determine all three edges), one
                 // set of atomics per triangle
@@ -597,14 +573,7 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
                     long long S1 = group_sum(grp, cnt, a1);
                     const int D0 = (int)__reduce_add_sync(grp, (unsigned)dq0);
                     const int D1 = (int)__reduce_add_sync(grp, (unsigned)dq1);
-                    if (lane == __ffs(grp) - 1) {
-                        long long S0, S2;
-                        ccw_from(S1, D0, D1, S0, S2);
-                        oriented(EG.w, S0, S1, S2);
-                        red_add(a.J + EG.x, S0);
-                        red_add(a.J + EG.y, S1);
-                        red_add(a.J + EG.z, S2);
-                    }
+                    if (lane == __ffs(grp) - 1) add_current(a, t0, S1, D0, D1);
                 }
                 // particles that leave go to this warp's ring (at most 31 + 32 entries)
                 const unsigned qmask = __ballot_sync(full, crossed);

@@ -301,6 +301,19 @@ struct alignas(sizeof(R) == 4 ? 128 : 64) TriRec {
                     // triangle's node k+2, its node entry+2 is node k+1)
 };
 
+// FP32 build: the currents of a step are summed per triangle and taken apart into edge
+// currents once, by the residual kernel.  With the local edges oriented counter-clockwise
+// (edge 0: 1->2, 1: 2->0, 2: 0->1) a segment s -> e in one triangle carries (Eq. current)
+//   A0 = s1 e2 - s2 e1,  A1 = s2 e0 - s0 e2,  A2 = s0 e1 - s1 e0,
+// and because s and e both sum to 2^22, the net outflow at each node is
+//   A2 - A1 = 2^22 (s0 - e0),  A0 - A2 = 2^22 (s1 - e1)   (the identity behind Eq. DCE),
+// so one product pair (A1) and two differences determine all three, also after summing
+// over the segments in the triangle; and the charge that leaves node k through the
+// triangle is the sum of s_k - e_k.
+struct alignas(32) FaceSum {
+    long long a1, d0, d1, pad;
+};
+
 struct PF32 {
     using R = float;
     using Lam = int32_t;
@@ -326,7 +339,7 @@ enum {
     CNT_ABSORBED = 0,
     CNT_OVERFLOW = 1,
     CNT_CROSSINGS = 2,
-    CNT_REMAINDER = 3,  // nodes where D_div J was not a multiple of 2^22 (must stay 0)
+    // 3: unused
     CNT_TIMEOUT = 4,    // bounded device waits that gave up (must stay 0)
     CNT_EMITTED = 5,    // particles born by the emitter
     CNT_NEXT_PID = 6,   // next particle id once an emitter was set
@@ -342,7 +355,8 @@ struct PushArgs {
     const TriRec<typename P::R> *rec;
     Particles<P> p;
     const int64_t *n_slots;     // device count of slots
-    typename P::Acc *J;         // N1, units: fixed 2^-44 (FP32) / 1 (FP64) of q_src/dt
+    typename P::Acc *J;         // FP64: N1 edge currents, units q_src/dt
+    FaceSum *face;              // FP32: N2 current sums, units 2^-44 and 2^-22 of q_src/dt
     typename P::Acc *Q;         // N0, Q^{n+1}, units 2^-22 / 1 of q_src
     typename P::Acc *Qabs;      // N0
     unsigned long long *counters;
@@ -427,9 +441,13 @@ struct FieldArgs {
     const typename P::R *loss_f;  // N2 x 2
     typename P::R *B;           // N2, B^{n-1/2} in, B^{n+1/2} out
     const typename P::R *mu_inv;// N2
-    const int32_t *edge_face;   // nf x 2, per free edge: (face+1) * sign, 0 if none
+    const int32_t *edge_face;   // N1 x 2, per edge: (4 face + local edge + 1) * sign, 0 if none
     const int32_t *free_edges;  // nf
-    typename P::Acc *J;         // N1 (zeroed by the face kernel before the particle step)
+    const int32_t *free_of_edge;// N1: index in free_edges or -1
+    // FP64: edge currents, zeroed by the face kernel before the particle step; FP32: written
+    // by the residual kernel from the triangles' sums, which the face kernel zeroes
+    typename P::Acc *J;
+    FaceSum *face;
     double *D;                  // N1 auxiliary dual flux (DGL)
     typename P::R *r;           // nf scratch: D_curl^T star_mu^-1 B - J
     // M in sliced ELL: slices of 32 rows, column-major inside a slice
@@ -440,9 +458,8 @@ struct FieldArgs {
     typename P::R dt;
     double j_scale;             // physical J = J_acc * j_scale
     // FP32 build: Q^{n+1} = Q^n - D_div J / 2^22 - Q_absorbed per node (exact)
-    const int64_t *node_ptr;    // N0 + 1: node -> incident edges
-    const int32_t *node_edge;
-    const int8_t *node_sign;    // +1 tail, -1 head
+    const int32_t *face_ptr;    // N0 + 1: node -> incident triangles
+    const int32_t *node_face;   // 4 triangle + local node
     const typename P::Acc *Qn;
     typename P::Acc *Qabs;      // N0 (zeroed by the face kernel before the particle step)
     typename P::Acc *Qnext;

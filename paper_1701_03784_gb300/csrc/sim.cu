@@ -132,7 +132,9 @@ struct SimImpl final : SimBase {
 
     TriRec<R> *rec = nullptr;
     R *E = nullptr, *B = nullptr, *mu_inv = nullptr, *r = nullptr;
-    int32_t *edge_face = nullptr, *free_edges = nullptr;
+    int32_t *edge_face = nullptr, *free_edges = nullptr, *free_of_edge = nullptr;
+    int32_t *face_ptr = nullptr, *node_face = nullptr;
+    FaceSum *face = nullptr;
     double *D = nullptr;
     int64_t *ell_off = nullptr;
     int32_t *ell_col = nullptr;
@@ -292,14 +294,28 @@ struct SimImpl final : SimBase {
         if ((st = upload(rec, hr)) != PIC_OK) return st;
         std::vector<R> hmu(mesh.mu_inv.begin(), mesh.mu_inv.end());
         if ((st = upload(mu_inv, hmu)) != PIC_OK) return st;
-        // the two faces of each free edge, in free-edge order
-        std::vector<int32_t> hef(2 * std::max<int64_t>(nf, 1), 0);
-        for (int64_t i = 0; i < nf; i++) {
-            const int64_t e = mesh.free_edges[i];
+        // the two faces of each edge, with the edge's place in them
+        std::vector<int32_t> hef(2 * mesh.N1, 0);
+        for (int64_t e = 0; e < mesh.N1; e++)
             for (int q2 = 0; q2 < 2; q2++) {
-                int32_t f = mesh.edge_face[2 * e + q2];
-                if (f >= 0) hef[2 * i + q2] = (f + 1) * mesh.edge_face_sign[2 * e + q2];
+                const int32_t f = mesh.edge_face[2 * e + q2];
+                if (f < 0) continue;
+                int k = 0;
+                while (mesh.tri_edge[3 * (int64_t)f + k] != e) k++;
+                hef[2 * e + q2] = (4 * f + k + 1) * mesh.edge_face_sign[2 * e + q2];
             }
+        if ((st = upload(free_of_edge, mesh.free_of_edge)) != PIC_OK) return st;
+        if constexpr (P::fixed) {
+            // the triangles of each node, with the node's place in them
+            std::vector<int32_t> fptr(mesh.N0 + 1, 0), nface(3 * mesh.N2);
+            for (int64_t k = 0; k < 3 * mesh.N2; k++) fptr[mesh.tri[k] + 1]++;
+            for (int64_t k = 0; k < mesh.N0; k++) fptr[k + 1] += fptr[k];
+            std::vector<int32_t> at(fptr.begin(), fptr.end() - 1);
+            for (int64_t f = 0; f < mesh.N2; f++)
+                for (int k = 0; k < 3; k++) nface[at[mesh.tri[3 * f + k]]++] = (int32_t)(4 * f + k);
+            if ((st = upload(face_ptr, fptr)) || (st = upload(node_face, nface)) ||
+                (st = dalloc(face, mesh.N2)))
+                return st;
         }
         if ((st = upload(edge_face, hef)) != PIC_OK) return st;
         if ((st = upload(free_edges, mesh.free_edges)) != PIC_OK) return st;
@@ -411,9 +427,10 @@ struct SimImpl final : SimBase {
         a.nf = nf;
         a.dt = (R)dt;
         a.j_scale = j_scale();
-        a.node_ptr = dd.node_ptr;
-        a.node_edge = dd.node_edge;
-        a.node_sign = dd.node_sign;
+        a.free_of_edge = free_of_edge;
+        a.face = face;
+        a.face_ptr = face_ptr;
+        a.node_face = node_face;
         a.Qn = nullptr;
         a.Qabs = Qabs;
         a.Qnext = nullptr;
@@ -1052,6 +1069,7 @@ struct SimImpl final : SimBase {
         pa.p = view;
         pa.n_slots = count;
         pa.J = J;
+        pa.face = face;
         pa.Q = Qbuf[1 - qcur];
         pa.Qabs = Qabs;
         pa.counters = counters;
@@ -1189,7 +1207,7 @@ struct SimImpl final : SimBase {
             o->sort_interval = sort_interval;
             o->n_steps = n_steps;
             o->dce_max = out[0];
-            o->dce_nonzero = (int64_t)out[1] + (int64_t)cnt[CNT_REMAINDER];
+            o->dce_nonzero = (int64_t)out[1];
             o->nr_dce_max = out[2];
             o->dgl_drift = out[3] / (out[4] > 0 ? out[4] : 1.0);
             o->field_energy = out[5];
