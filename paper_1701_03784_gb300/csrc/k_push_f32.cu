@@ -239,10 +239,9 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, unsigned b
 // producer lane: stage tile `tile` (slots [tile*TILE, tile*TILE + TILE) clipped to n, rounded up
 // to 4 slots so every copy is a multiple of 16 bytes; the arrays have that much room)
 __device__ __forceinline__ void issue_tile(const PushArgs<PF32> &a, PushSmem &sm, int stage,
-                                           long long tile, long long n) {
-    const long long base = tile * TILE;
-    const long long cnt = min((long long)TILE, n - base);
-    const unsigned bytes = (unsigned)(((cnt + 3) & ~3LL) * 4);
+                                           int tile, unsigned n) {
+    const unsigned base = (unsigned)tile * TILE, cnt = min((unsigned)TILE, n - base);
+    const unsigned bytes = ((cnt + 3) & ~3u) * 4;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     unsigned long long *bar = &sm.full[stage];
     mbar_expect_tx(bar, 6 * bytes);
@@ -505,22 +504,34 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
     }
     __syncthreads();
     chain_wait();
-    const long long n = *a.n_slots;
-    const long long ntiles = (n + TILE - 1) / TILE;
-    // each CTA takes a contiguous range of tiles: consecutive tiles hold neighbouring
-    // triangles (slots are sorted by triangle), so their records stay in this SM's L1
-    const long long per = (ntiles + gridDim.x - 1) / gridDim.x;
-    const long long tile0 = (long long)blockIdx.x * per, tile1 = min(ntiles, tile0 + per);
-    if (tile0 >= tile1) return;
+    // slot numbers fit 31 bits (the capacity's limit); sums past the last slot 32
+    const unsigned n = (unsigned)a.n_slots[0];
+    const int ntiles = (int)((n + (TILE - 1)) / TILE);
+    // each CTA takes a contiguous range of the tiles that the last re-sort ordered:
+    // consecutive tiles hold neighbouring triangles, so their records stay in this SM's L1.
+    // Tiles of births since then hold particles of many triangles, whose sums a warp takes
+    // one after another: they are dealt out singly, from the last CTA on (as the end of
+    // the contiguous ranges, 32,000 of a diode's 4M particles kept five CTAs busy three
+    // times as long as all the others: 195 us a launch).
+    const unsigned ordered = a.sorted ? n : min(n, (unsigned)a.n_slots[1]);
+    const int otiles = (int)((ordered + (TILE - 1)) / TILE), grid = (int)gridDim.x;
+    // runs differ by at most a tile: equal ones left a sixth of the CTAs idle at 977 tiles
+    const int per = otiles / grid, more = otiles % grid, b = (int)blockIdx.x;
+    const int tile0 = b * per + min(b, more), run = per + (b < more ? 1 : 0);
+    const int deal = otiles + (grid - 1 - b);
+    const int count = run + (deal < ntiles ? (ntiles - 1 - deal) / grid + 1 : 0);
+    if (count <= 0) return;
+    const int first = run > 0 ? tile0 : deal;
+    const auto after = [&](int tile, int it) { return it + 1 < run ? tile + 1 : it + 1 == run ? deal : tile + grid; };
     unsigned cx = 0;
 
     if (warp == CW) {
         // ---- producer warp: lane 0 stages the CTA's tiles; a stage is refilled once every
         // compute warp has released its previous tile
         if (lane == 0) {
-            long long it = 0;
-            for (long long tile = tile0; tile < tile1; tile++, it++) {
-                const int stage = (int)(it % STAGES);
+            int it = 0;
+            for (int tile = first; it < count; tile = after(tile, it), it++) {
+                const int stage = it % STAGES;
                 if (it >= STAGES &&
                     !mbar_wait(&sm.empty[stage], (unsigned)((it / STAGES - 1) & 1), a.wait_polls)) {
                     atomicAdd(a.counters + CNT_TIMEOUT, 1ULL);
@@ -532,8 +543,8 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
             // landed: wait (bounded) for the last phase issued on each stage.  After a
             // normal run the compute warps have seen these phases and the waits return at
             // once; after a timeout they may not have.
-            for (long long k = it > STAGES ? it - STAGES : 0; k < it; k++)
-                if (!mbar_wait(&sm.full[(int)(k % STAGES)], (unsigned)((k / STAGES) & 1)))
+            for (int k = it > STAGES ? it - STAGES : 0; k < it; k++)
+                if (!mbar_wait(&sm.full[k % STAGES], (unsigned)((k / STAGES) & 1)))
                     atomicAdd(a.counters + CNT_TIMEOUT, 1ULL);
         }
     } else {
@@ -542,9 +553,8 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
         QEntry *ring = sm.q[warp];
         const unsigned below = (1u << lane) - 1;
         unsigned head = 0, tail = 0;   // warp-uniform, ring index = value & (QCAP - 1)
-        long long it = 0;
-        for (long long tile = tile0; tile < tile1; tile++, it++) {
-            const int stage = (int)(it % STAGES);
+        for (int it = 0, tile = first; it < count; tile = after(tile, it), it++) {
+            const int stage = it % STAGES;
             const bool ok = mbar_wait(&sm.full[stage], (unsigned)((it / STAGES) & 1), a.wait_polls);
             if (__any_sync(full, !ok)) {
                 // leave; the producer drains the copies in flight before the block exits
@@ -552,10 +562,10 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
                 break;
             }
             const TileBuf &b = sm.buf[stage];
-            const long long base = tile * TILE;
+            const unsigned base = (unsigned)tile * TILE;
             for (int r = 0; r < ROUNDS; r++) {
                 const int k = r * PT + tid;
-                const long long i = base + k;
+                const unsigned i = base + (unsigned)k;
                 const int t0 = i < n ? b.tri[k] : -1;
                 long long a1 = 0;
                 int dq0 = 0, dq1 = 0;

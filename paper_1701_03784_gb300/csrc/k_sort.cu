@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(256) k_scan_top(int32_t *blk, int64_t nblk, in
         if (threadIdx.x == 255) carry += sh[255];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *n_slots = carry;
+    if (threadIdx.x == 0) n_slots[0] = n_slots[1] = carry;
 }
 
 // exclusive scan inside each chunk plus the chunk's offset; the result is the write

@@ -354,7 +354,10 @@ template <class P>
 struct PushArgs {
     const TriRec<typename P::R> *rec;
     Particles<P> p;
-    const int64_t *n_slots;     // device count of slots
+    // device count of slots; behind it how many of them the last re-sort ordered (births
+    // since then follow them), unless `sorted` says that all are in order
+    const int64_t *n_slots;
+    bool sorted = false;
     typename P::Acc *J;         // FP64: N1 edge currents, units q_src/dt
     FaceSum *face;              // FP32: N2 current sums, units 2^-44 and 2^-22 of q_src/dt
     typename P::Acc *Q;         // N0, Q^{n+1}, units 2^-22 / 1 of q_src
@@ -489,7 +492,7 @@ struct SortScratch {
     int64_t *n_old = nullptr;    // slot count before the sort
 };
 // stable-enough counting sort by triangle; drops removed particles; writes the new
-// slot count to *n_slots (device)
+// slot count to n_slots[0] and n_slots[1] (device)
 template <class P>
 void launch_resort(Particles<P> src, Particles<P> dst, int64_t *n_slots, int64_t n_bound,
                    int64_t N2, const SortScratch &sc, cudaStream_t s);

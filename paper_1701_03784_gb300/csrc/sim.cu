@@ -142,7 +142,7 @@ struct SimImpl final : SimBase {
     Acc *J = nullptr, *Qbuf[2] = {nullptr, nullptr}, *Qabs = nullptr, *qpos = nullptr;
     Acc *Qwall = nullptr;   // charge removed at walls since the Gauss-law reference
     Particles<P> parts[2];
-    int64_t *d_n = nullptr;
+    int64_t *d_n = nullptr;   // slots, and how many of them the last re-sort ordered
     unsigned long long *counters = nullptr;
     SortScratch sc;
     DiagDev dd{};
@@ -362,9 +362,9 @@ struct SimImpl final : SimBase {
                 return st;
         }
         // the diagnostics' results behind the counters: one copy reads both
-        if ((st = dalloc(d_n, 1)) || (st = dalloc(counters, CNT_N + 8))) return st;
+        if ((st = dalloc(d_n, 2)) || (st = dalloc(counters, CNT_N + 8))) return st;
         diag_out = reinterpret_cast<double *>(counters + CNT_N);
-        PIC_CUDA_TRY(cudaMemset(d_n, 0, sizeof(int64_t)));
+        PIC_CUDA_TRY(cudaMemset(d_n, 0, 2 * sizeof(int64_t)));
         PIC_CUDA_TRY(cudaMemset(counters, 0, sizeof(unsigned long long) * CNT_N));
         // sort scratch
         if ((st = dalloc(sc.cnt, mesh.N2 + 1)) || (st = dalloc(sc.blk, mesh.N2 / 2048 + 2)) ||
@@ -761,6 +761,13 @@ struct SimImpl final : SimBase {
         return PIC_OK;
     }
 
+    // n slots, all taken to be in order
+    pic_status set_count(int64_t n, cudaStream_t s) {
+        const int64_t both[2] = {n, n};
+        PIC_CUDA_TRY(cudaMemcpyAsync(d_n, both, sizeof both, cudaMemcpyHostToDevice, s));
+        return PIC_OK;
+    }
+
     pic_status read_count(int64_t *n, cudaStream_t s) {
         PIC_CUDA_TRY(cudaMemcpyAsync(n, d_n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         PIC_CUDA_TRY(cudaStreamSynchronize(s));
@@ -859,8 +866,8 @@ struct SimImpl final : SimBase {
         PIC_CUDA_TRY(cudaMemcpyAsync(p.up + n_now, vp.data(), sizeof(R) * n, cudaMemcpyHostToDevice, s));
         PIC_CUDA_TRY(cudaMemcpyAsync(p.uz + n_now, vz.data(), sizeof(R) * n, cudaMemcpyHostToDevice, s));
         PIC_CUDA_TRY(cudaMemcpyAsync(p.pid + n_now, pid.data(), 4 * n, cudaMemcpyHostToDevice, s));
-        int64_t n_new = n_now + n;
-        PIC_CUDA_TRY(cudaMemcpyAsync(d_n, &n_new, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        const int64_t n_new = n_now + n;
+        if ((st = set_count(n_new, s)) != PIC_OK) return st;
         launch_deposit_q<P>(rec, p, n_now, n, nullptr, Qn(), s);
         n_bound = emitting ? cap : n_new;
         next_pid += n;
@@ -1357,7 +1364,7 @@ struct SimImpl final : SimBase {
         pic_status st = copy_slots(const_cast<char *>(static_cast<const char *>(src)), n, 0, n,
                                    true, s);
         if (st != PIC_OK) return st;
-        PIC_CUDA_TRY(cudaMemcpyAsync(d_n, &n, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        if ((st = set_count(n, s)) != PIC_OK) return st;
         n_bound = emitting ? cap : n;
         dgl_dirty = true;
         return PIC_OK;
@@ -1410,6 +1417,7 @@ struct SimImpl final : SimBase {
                 v.pid += c0;
                 PushArgs<P> pa = push_args(v, d_chunk_n + c);
                 pa.chain = false;   // it follows the upload's event
+                pa.sorted = true;
                 launch_push<P>(pa, c1 - c0, s);
             }
             if (!resort_due) {
@@ -1486,7 +1494,7 @@ struct SimImpl final : SimBase {
             PIC_CUDA_TRY(cudaStreamWaitEvent(s, rt_up, 0));
             if (k == 0) {
                 // the caller's state: its slot count, and a new Gauss-law reference
-                PIC_CUDA_TRY(cudaMemcpyAsync(d_n, &n, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+                if ((st = set_count(n, s)) != PIC_OK) return st;
                 n_bound = emitting ? cap : n;
                 dgl_dirty = true;
             }
