@@ -425,7 +425,7 @@ pic_status pic_particles_raw_set(pic_sim *s, const void *host_src, int64_t n_slo
  * every step uploads it, steps, and writes it back.  Slots beyond the live count after a
  * re-sort removed particles are unspecified on return.  Uploads and downloads run on
  * internal streams, chunk by chunk: the download of one step overlaps the upload of the
- * next, and (FP32 build, kernel timing off) after the first step the particle kernel runs
+ * next, and (FP32 build, kernel timing off) the particle kernel runs
  * on each chunk as soon as it has landed and each chunk is written back as soon as it is
  * pushed (after the re-sort, on a re-sort step); the result is bit-identical to stepping
  * on the device.  The call is asynchronous on cuda_stream, which waits for the last

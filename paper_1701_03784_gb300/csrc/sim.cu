@@ -5,6 +5,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 
 #include "pic_internal.h"
 
@@ -125,7 +126,7 @@ struct SimImpl final : SimBase {
     std::vector<void *> allocs;
     double dt = 0, bz = 0, q = 0, mass = 0, weight = 0, q_src = 0, qm = 0;
     bool have_species = false;
-    int64_t cap = 0, n_bound = 0, next_pid = 0, n_steps = 0, n_injected = 0;
+    int64_t cap = 0, pitch = 0, n_bound = 0, next_pid = 0, n_steps = 0, n_injected = 0;
     int cur = 0, qcur = 0, since_sort = 0;
     bool dgl_dirty = true;
     int64_t nf = 0, n_slices = 0;
@@ -173,10 +174,9 @@ struct SimImpl final : SimBase {
 
     bool timing_on = false;
     // host round trips (step_host): uploads and downloads run on streams of their own,
-    // chunk by chunk (16M slots, ms per step: 2, 3, 4, 6, 8, 16, 32 chunks -> 2.63, 2.53,
-    // 2.57, 2.66, 2.75, 3.15, 3.15; each chunk costs a particle-kernel launch and six
-    // copies each way, more than the shorter pipeline tail saves)
-    static constexpr int RT_CHUNKS = 3;
+    // chunk by chunk (8M slots, ms for four steps: 3, 4, 6 chunks -> 5.56, 5.53, 5.55; fewer
+    // leave a longer pipeline to fill and drain, more pay for launches and copies)
+    static constexpr int RT_CHUNKS = 4;
     // CUDA-graph replay of whole periods of steps (2 x the re-sort interval: the buffer
     // parities and the re-sort phase are back where they started)
     bool use_graph = false, stepped = false;
@@ -352,14 +352,24 @@ struct SimImpl final : SimBase {
         PIC_CUDA_TRY(cudaMemset(J, 0, sizeof(Acc) * mesh.N1));
         for (int k = 0; k < 2; k++) PIC_CUDA_TRY(cudaMemset(Qbuf[k], 0, sizeof(Acc) * mesh.N0));
         PIC_CUDA_TRY(cudaMemset(Qabs, 0, sizeof(Acc) * mesh.N0));
-        // particles, double-buffered for the re-sort
+        // particles, double-buffered for the re-sort; each buffer one allocation, its arrays at
+        // a common distance in the FP32 build (host round trips copy them as rows)
+        pitch = (cap + SLOT_PAD + 63) / 64 * 64;   // bulk copies round up to 16 bytes
         for (int k = 0; k < 2; k++) {
             Particles<P> &p = parts[k];
-            const int64_t ca = cap + SLOT_PAD;  // bulk copies round up to 16 bytes
-            if ((st = dalloc(p.tri, ca)) || (st = dalloc(p.l0, ca)) || (st = dalloc(p.l1, ca)) ||
-                (st = dalloc(p.ur, ca)) || (st = dalloc(p.up, ca)) || (st = dalloc(p.uz, ca)) ||
-                (st = dalloc(p.pid, ca)))
-                return st;
+            char *at = nullptr;
+            if ((st = dalloc(at, pitch * (8 + 2 * (int64_t)sizeof(Lam) + 3 * (int64_t)sizeof(R))))) return st;
+            const auto take = [&](auto *&x) {
+                x = reinterpret_cast<std::remove_reference_t<decltype(x)>>(at);
+                at += sizeof(*x) * pitch;
+            };
+            take(p.tri);
+            take(p.l0);
+            take(p.l1);
+            take(p.ur);
+            take(p.up);
+            take(p.uz);
+            take(p.pid);
         }
         // the diagnostics' results behind the counters: one copy reads both
         if ((st = dalloc(d_n, 2)) || (st = dalloc(counters, CNT_N + 8))) return st;
@@ -1370,10 +1380,21 @@ struct SimImpl final : SimBase {
         return PIC_OK;
     }
 
-    // slots [c0, c1) of the raw state, host <-> device (one copy per array; array k starts
-    // at sum_{j<k} size_j * raw_stride(n) bytes of the host buffer)
+    // slots [c0, c1) of the raw state, host <-> device (array k starts at
+    // sum_{j<k} size_j * raw_stride(n) bytes of the host buffer): in the FP32 build the six
+    // arrays as the rows of one copy, as far as CUDA takes such strides (six copies a chunk
+    // and direction took four steps on 8M slots 6.08 ms)
     pic_status copy_slots(char *h, int64_t n, int64_t c0, int64_t c1, bool up, cudaStream_t s) {
         const Particles<P> &p = parts[cur];
+        const size_t dp = 4 * (size_t)pitch, hp = 4 * (size_t)raw_stride(n);
+        if (P::fixed && dp < ((size_t)1 << 31) && hp < ((size_t)1 << 31)) {
+            char *d = reinterpret_cast<char *>(p.tri) + 4 * c0, *hk = h + 4 * c0;
+            const size_t w = 4 * (size_t)(c1 - c0);
+            if (w == 0) return PIC_OK;
+            if (up) PIC_CUDA_TRY(cudaMemcpy2DAsync(d, dp, hk, hp, w, 6, cudaMemcpyHostToDevice, s));
+            else PIC_CUDA_TRY(cudaMemcpy2DAsync(hk, hp, d, dp, w, 6, cudaMemcpyDeviceToHost, s));
+            return PIC_OK;
+        }
         void *dev[6] = {p.tri, p.l0, p.l1, p.ur, p.up, p.uz};
         const size_t sz[6] = {4, sizeof(Lam), sizeof(Lam), sizeof(R), sizeof(R), sizeof(R)};
         for (int k = 0; k < 6; k++) {
@@ -1391,7 +1412,7 @@ struct SimImpl final : SimBase {
     // copies: chunk c is uploaded once the previous step's write-back of it is done,
     // pushed once it has landed, and written back once it is pushed (or, on a re-sort
     // step, once the re-sort is done)
-    pic_status step_host_pipelined(char *h, int64_t n, int64_t chunk, cudaStream_t s) {
+    pic_status step_host_pipelined(char *h, int64_t n, int64_t chunk, bool first, cudaStream_t s) {
         pic_status st;
         stepped = true;
         FieldArgs<P> fa = field_args();
@@ -1402,7 +1423,7 @@ struct SimImpl final : SimBase {
         const bool resort_due = sort_interval > 0 && since_sort + 1 >= sort_interval;
         for (int c = 0; c < RT_CHUNKS; c++) {
             const int64_t c0 = std::min(n, c * chunk), c1 = std::min(n, c0 + chunk);
-            PIC_CUDA_TRY(cudaStreamWaitEvent(up_stream, rt_chunk[c], 0));
+            if (!first) PIC_CUDA_TRY(cudaStreamWaitEvent(up_stream, rt_chunk[c], 0));
             if (c1 > c0 && (st = copy_slots(h, n, c0, c1, true, up_stream)) != PIC_OK) return st;
             PIC_CUDA_TRY(cudaEventRecord(rt_upc[c], up_stream));
             PIC_CUDA_TRY(cudaStreamWaitEvent(s, rt_upc[c], 0));
@@ -1466,11 +1487,12 @@ struct SimImpl final : SimBase {
         // chunks of whole particle-kernel tiles (512 slots), so that a chunk's tiles read
         // none of the next chunk's slots
         const int64_t chunk = ((n + RT_CHUNKS - 1) / RT_CHUNKS + 511) / 512 * 512;
-        // FP32 build (without kernel timing): after the first step each chunk is pushed as
-        // soon as it has landed and written back as soon as it is pushed, so the step's
-        // particle work overlaps both copy directions; the E update and any re-sort follow
-        // the last chunk (a re-sort moves slots between chunks: then the write-back waits
-        // for it)
+        // FP32 build (without kernel timing): each chunk is pushed as soon as it has landed and
+        // written back as soon as it is pushed, so the step's particle work overlaps both
+        // copy directions; the E update and any re-sort follow the last chunk (a re-sort
+        // moves slots between chunks: then the write-back waits for it).  With the first
+        // step outside this (uploaded whole, stepped, then written back), four steps on 8M
+        // slots took 6.63 ms.
         const bool pipe = P::fixed && !timing_on;
         pic_status st;
         if (pipe && !d_chunk_n && (st = dalloc(d_chunk_n, RT_CHUNKS)) != PIC_OK) return st;
@@ -1478,8 +1500,14 @@ struct SimImpl final : SimBase {
         PIC_CUDA_TRY(cudaEventRecord(rt_up, s));
         PIC_CUDA_TRY(cudaStreamWaitEvent(up_stream, rt_up, 0));
         for (int64_t k = 0; k < steps; k++) {
-            if (k > 0 && pipe) {
-                if ((st = step_host_pipelined(h, n, chunk, s)) != PIC_OK) return st;
+            if (pipe) {
+                if (k == 0) {
+                    // the caller's state: its slot count, and a new Gauss-law reference
+                    if ((st = set_count(n, s)) != PIC_OK) return st;
+                    n_bound = n;
+                    dgl_dirty = true;
+                }
+                if ((st = step_host_pipelined(h, n, chunk, k == 0, s)) != PIC_OK) return st;
                 continue;
             }
             // upload; chunk c waits only for the previous step's download of chunk c, so the
