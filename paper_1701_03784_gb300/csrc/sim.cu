@@ -262,48 +262,50 @@ struct SimImpl final : SimBase {
         pic_status st;
         // triangle records
         std::vector<TriRec<R>> hr(mesh.N2);
-        for (int64_t t = 0; t < mesh.N2; t++) {
-            TriRec<R> &x = hr[t];
-            std::memset(&x, 0, sizeof x);
-            for (int k = 0; k < 4; k++) x.g[k] = (R)mesh.grad[6 * t + k];
-            int flags = 0;
-            for (int k = 0; k < 3; k++) {
-                int32_t nk = mesh.tri[3 * t + k];
-                x.node[k] = nk;
-                x.rho[k] = (R)mesh.zr[2 * nk + 1];
-                x.edge[k] = mesh.tri_edge[3 * t + k];
-                int32_t nb = mesh.tri_nbr[3 * t + k];
-                x.nbr[k] = nb >= 0 ? nb : -mesh.edge_tag[mesh.tri_edge[3 * t + k]];
-                if (mesh.tri[3 * t + (k + 1) % 3] < mesh.tri[3 * t + (k + 2) % 3]) flags |= 1 << k;
-            }
-            x.flags = flags;
-            x.eflags = flags;
-            int entry = 0;
-            for (int k = 0; k < 3; k++) {
-                const int32_t nb = mesh.tri_nbr[3 * t + k];
-                if (nb < 0) continue;
-                const int32_t ga = mesh.tri[3 * t + (k + 1) % 3], gb = mesh.tri[3 * t + (k + 2) % 3];
-                for (int j = 0; j < 3; j++) {
-                    const int32_t q = mesh.tri[3 * nb + j];
-                    if (q != ga && q != gb) entry |= j << (2 * k);
+        parallel_for(mesh.N2, [&](int64_t t_a, int64_t t_b) {
+            for (int64_t t = t_a; t < t_b; t++) {
+                TriRec<R> &x = hr[t];
+                std::memset(&x, 0, sizeof x);
+                for (int k = 0; k < 4; k++) x.g[k] = (R)mesh.grad[6 * t + k];
+                int flags = 0;
+                for (int k = 0; k < 3; k++) {
+                    int32_t nk = mesh.tri[3 * t + k];
+                    x.node[k] = nk;
+                    x.rho[k] = (R)mesh.zr[2 * nk + 1];
+                    x.edge[k] = mesh.tri_edge[3 * t + k];
+                    int32_t nb = mesh.tri_nbr[3 * t + k];
+                    x.nbr[k] = nb >= 0 ? nb : -mesh.edge_tag[mesh.tri_edge[3 * t + k]];
+                    if (mesh.tri[3 * t + (k + 1) % 3] < mesh.tri[3 * t + (k + 2) % 3]) flags |= 1 << k;
                 }
+                x.flags = flags;
+                x.eflags = flags;
+                int entry = 0;
+                for (int k = 0; k < 3; k++) {
+                    const int32_t nb = mesh.tri_nbr[3 * t + k];
+                    if (nb < 0) continue;
+                    const int32_t ga = mesh.tri[3 * t + (k + 1) % 3], gb = mesh.tri[3 * t + (k + 2) % 3];
+                    for (int j = 0; j < 3; j++) {
+                        const int32_t q = mesh.tri[3 * nb + j];
+                        if (q != ga && q != gb) entry |= j << (2 * k);
+                    }
+                }
+                x.entry = entry;
+                x.inv_area = (R)(1.0 / mesh.area[t]);
             }
-            x.entry = entry;
-            x.inv_area = (R)(1.0 / mesh.area[t]);
-        }
+        });
         if ((st = upload(rec, hr)) != PIC_OK) return st;
         std::vector<R> hmu(mesh.mu_inv.begin(), mesh.mu_inv.end());
         if ((st = upload(mu_inv, hmu)) != PIC_OK) return st;
         // the two faces of each edge, with the edge's place in them
         std::vector<int32_t> hef(2 * mesh.N1, 0);
-        for (int64_t e = 0; e < mesh.N1; e++)
-            for (int q2 = 0; q2 < 2; q2++) {
-                const int32_t f = mesh.edge_face[2 * e + q2];
-                if (f < 0) continue;
-                int k = 0;
-                while (mesh.tri_edge[3 * (int64_t)f + k] != e) k++;
-                hef[2 * e + q2] = (4 * f + k + 1) * mesh.edge_face_sign[2 * e + q2];
-            }
+        parallel_for(mesh.N2, [&](int64_t f_a, int64_t f_b) {
+            for (int64_t f = f_a; f < f_b; f++)
+                for (int k = 0; k < 3; k++) {
+                    const int64_t e = mesh.tri_edge[3 * f + k];
+                    const int64_t q2 = 2 * e + (mesh.edge_face[2 * e] == f ? 0 : 1);
+                    hef[q2] = (int32_t)(4 * f + k + 1) * mesh.edge_face_sign[q2];
+                }
+        });
         if ((st = upload(free_of_edge, mesh.free_of_edge)) != PIC_OK) return st;
         if constexpr (P::fixed) {
             // the triangles of each node, with the node's place in them
@@ -330,13 +332,15 @@ struct SimImpl final : SimBase {
         }
         std::vector<int32_t> hcol(std::max<int64_t>(hoff[n_slices], 1), 0);
         std::vector<R> hval(std::max<int64_t>(hoff[n_slices], 1), R(0));
-        for (int64_t i = 0; i < nf; i++) {
-            int64_t sl = i / 32, lane = i % 32, k = 0;
-            for (int64_t q2 = mesh.M_ptr[i]; q2 < mesh.M_ptr[i + 1]; q2++, k++) {
-                hcol[hoff[sl] + 32 * k + lane] = mesh.M_idx[q2];
-                hval[hoff[sl] + 32 * k + lane] = (R)mesh.M_val[q2];
+        parallel_for(nf, [&](int64_t i_a, int64_t i_b) {
+            for (int64_t i = i_a; i < i_b; i++) {
+                int64_t sl = i / 32, lane = i % 32, k = 0;
+                for (int64_t q2 = mesh.M_ptr[i]; q2 < mesh.M_ptr[i + 1]; q2++, k++) {
+                    hcol[hoff[sl] + 32 * k + lane] = mesh.M_idx[q2];
+                    hval[hoff[sl] + 32 * k + lane] = (R)mesh.M_val[q2];
+                }
             }
-        }
+        });
         if ((st = upload(ell_off, hoff)) != PIC_OK) return st;
         if ((st = upload(ell_col, hcol)) != PIC_OK) return st;
         if ((st = upload(ell_val, hval)) != PIC_OK) return st;
@@ -1202,8 +1206,13 @@ struct SimImpl final : SimBase {
             dst[ra.count] = to;
             ra.add(f, x, scale, n);
         };
-        want(Eo, E, nullptr, 1.0, m->N1);
-        want(Bo, B, nullptr, 1.0, m->N2);
+        if constexpr (P::fixed) {
+            want(Eo, E, nullptr, 1.0, m->N1);
+            want(Bo, B, nullptr, 1.0, m->N2);
+        } else {
+            if (Eo) PIC_CUDA_TRY(cudaMemcpyAsync(Eo, E, sizeof(R) * m->N1, cudaMemcpyDeviceToHost, s));
+            if (Bo) PIC_CUDA_TRY(cudaMemcpyAsync(Bo, B, sizeof(R) * m->N2, cudaMemcpyDeviceToHost, s));
+        }
         want(Jo, nullptr, J, j_scale(), m->N1);
         pic_status st = read_arrays(ra, dst, s);
         PIC_CUDA_TRY(cudaStreamSynchronize(s));   // also before leaving with an error: res is ours
