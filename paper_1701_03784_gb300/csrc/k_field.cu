@@ -63,8 +63,11 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
         if constexpr (P::fixed) mu = a.mu_inv[f];
     }
     chain_wait();
-    if constexpr (!P::fixed)
+    if constexpr (!P::fixed) {
         if (f < a.N1) a.J[f] = 0;
+    } else if (f == 0) {
+        a.counters[CNT_TILE] = 0;
+    }
     if (f < a.N0) {
         a.Qabs[f] = 0;
         if constexpr (!P::fixed) a.Qnext[f] = 0;

@@ -49,6 +49,7 @@ constexpr int NT = PT + 32;        // plus one producer warp
 constexpr int ROUNDS = 2;          // slots per compute thread per tile
 constexpr int TILE = PT * ROUNDS;  // slots per tile
 constexpr int STAGES = 2;          // tile buffers in flight
+constexpr int SHARE = 4;           // one tile in SHARE of long runs is taken singly (see below)
 constexpr int QCAP = 64;           // ring entries per compute warp (at most 31 + 32 used)
 constexpr unsigned WAIT_SLICE_NS = 100000;    // one bounded mbarrier poll sleeps <= 100 us
 constexpr long long WAIT_LIMIT = PUSH_WAIT_POLLS;   // polls of a drain wait (<= ~1.6 s)
@@ -194,6 +195,7 @@ struct PushSmem {
     QEntry q[CW][QCAP];                // per compute warp: ring of particles to walk on
     unsigned long long full[STAGES];   // the bulk copies of a stage's tile landed
     unsigned long long empty[STAGES];  // every compute warp released the stage
+    int tile[STAGES];                  // which tile a stage holds; -1: no more
 };
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
@@ -507,22 +509,27 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
     // slot numbers fit 31 bits (the capacity's limit); sums past the last slot 32
     const unsigned n = (unsigned)a.n_slots[0];
     const int ntiles = (int)((n + (TILE - 1)) / TILE);
-    // each CTA takes a contiguous range of the tiles that the last re-sort ordered:
-    // consecutive tiles hold neighbouring triangles, so their records stay in this SM's L1.
-    // Tiles of births since then hold particles of many triangles, whose sums a warp takes
-    // one after another: they are dealt out singly, from the last CTA on (as the end of
-    // the contiguous ranges, 32,000 of a diode's 4M particles kept five CTAs busy three
-    // times as long as all the others: 195 us a launch).
+    // Each CTA takes a run of the tiles that the last re-sort ordered: consecutive tiles hold
+    // neighbouring triangles, so their records stay in this SM's L1.  Runs differ by at most
+    // a tile (equal ones left a sixth of the CTAs idle at 977 tiles).  What follows is taken
+    // tile by tile by whoever is free, through a counter:
+    //  * tiles of births since the re-sort, first: their triangles are mixed, and a warp takes
+    //    the sums of its triangles one after another (at the end of the runs, 32,000 of a
+    //    diode's 4M particles kept five CTAs busy three times as long as all the others:
+    //    195 us a launch instead of 99);
+    //  * where the runs are long, the last SHARE-th of the ordered tiles: with runs alone the
+    //    SMs were done between 493k and 545k of a launch's 551k cycles (16M particles), and
+    //    a launch took 254 us; with one tile in 16, 8, 4, 3, 2 taken singly 252, 245, 245,
+    //    248, 252 (the diode's 97, 90, 82, 79, 80).
+    // (Launches on a range of the slots share the step, so they keep to runs.)
     const unsigned ordered = a.sorted ? n : min(n, (unsigned)a.n_slots[1]);
     const int otiles = (int)((ordered + (TILE - 1)) / TILE), grid = (int)gridDim.x;
-    // runs differ by at most a tile: equal ones left a sixth of the CTAs idle at 977 tiles
-    const int per = otiles / grid, more = otiles % grid, b = (int)blockIdx.x;
+    const int shared = a.sorted || otiles < SHARE * grid ? 0 : otiles / SHARE;
+    const int runs = otiles - shared;
+    const int per = runs / grid, more = runs % grid, b = (int)blockIdx.x;
     const int tile0 = b * per + min(b, more), run = per + (b < more ? 1 : 0);
-    const int deal = otiles + (grid - 1 - b);
-    const int count = run + (deal < ntiles ? (ntiles - 1 - deal) / grid + 1 : 0);
-    if (count <= 0) return;
-    const int first = run > 0 ? tile0 : deal;
-    const auto after = [&](int tile, int it) { return it + 1 < run ? tile + 1 : it + 1 == run ? deal : tile + grid; };
+    const int births = ntiles - otiles, open = births + shared;
+    if (run + open <= 0) return;
     unsigned cx = 0;
 
     if (warp == CW) {
@@ -530,20 +537,32 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
         // compute warp has released its previous tile
         if (lane == 0) {
             int it = 0;
-            for (int tile = first; it < count; tile = after(tile, it), it++) {
+            bool ended = false;
+            for (;; it++) {
+                int tile = tile0 + it;
+                if (it >= run) {
+                    const int d = open > 0 ? (int)atomicAdd(a.counters + CNT_TILE, 1ULL) : 0;
+                    tile = d >= open ? -1 : d < births ? otiles + d : runs + (d - births);
+                }
                 const int stage = it % STAGES;
                 if (it >= STAGES &&
                     !mbar_wait(&sm.empty[stage], (unsigned)((it / STAGES - 1) & 1), a.wait_polls)) {
                     atomicAdd(a.counters + CNT_TIMEOUT, 1ULL);
                     break;
                 }
+                sm.tile[stage] = tile;
+                if (tile < 0) {
+                    mbar_arrive(&sm.full[stage]);   // no more
+                    ended = true;
+                    break;
+                }
                 issue_tile(a, sm, stage, tile, n);
             }
             // before the block can exit, every copy issued into its shared memory has
-            // landed: wait (bounded) for the last phase issued on each stage.  After a
-            // normal run the compute warps have seen these phases and the waits return at
-            // once; after a timeout they may not have.
-            for (int k = it > STAGES ? it - STAGES : 0; k < it; k++)
+            // landed: wait (bounded) for the last phase issued on each stage (the stage that
+            // took the end mark had been released: its copy was seen).  After a normal run
+            // the waits return at once; after a timeout they may not.
+            for (int k = max(it - STAGES + (ended ? 1 : 0), 0); k < it; k++)
                 if (!mbar_wait(&sm.full[k % STAGES], (unsigned)((k / STAGES) & 1)))
                     atomicAdd(a.counters + CNT_TIMEOUT, 1ULL);
         }
@@ -553,7 +572,7 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
         QEntry *ring = sm.q[warp];
         const unsigned below = (1u << lane) - 1;
         unsigned head = 0, tail = 0;   // warp-uniform, ring index = value & (QCAP - 1)
-        for (int it = 0, tile = first; it < count; tile = after(tile, it), it++) {
+        for (int it = 0;; it++) {
             const int stage = it % STAGES;
             const bool ok = mbar_wait(&sm.full[stage], (unsigned)((it / STAGES) & 1), a.wait_polls);
             if (__any_sync(full, !ok)) {
@@ -561,6 +580,8 @@ __global__ void __launch_bounds__(NT, 4) k_push_f32(const __grid_constant__ Push
                 if (lane == 0) atomicAdd(a.counters + CNT_TIMEOUT, 1ULL);
                 break;
             }
+            const int tile = sm.tile[stage];
+            if (tile < 0) break;
             const TileBuf &b = sm.buf[stage];
             const unsigned base = (unsigned)tile * TILE;
             for (int r = 0; r < ROUNDS; r++) {

@@ -339,7 +339,7 @@ enum {
     CNT_ABSORBED = 0,
     CNT_OVERFLOW = 1,
     CNT_CROSSINGS = 2,
-    // 3: unused
+    CNT_TILE = 3,       // FP32 particle kernel: tiles taken so far from the shared end (zeroed per step)
     CNT_TIMEOUT = 4,    // bounded device waits that gave up (must stay 0)
     CNT_EMITTED = 5,    // particles born by the emitter
     CNT_NEXT_PID = 6,   // next particle id once an emitter was set
