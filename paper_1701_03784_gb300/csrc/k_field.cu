@@ -109,6 +109,14 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
     for (int k = 0; k < 8; k += W) *reinterpret_cast<R4 *>(out + k) = *reinterpret_cast<R4 *>(w + k);
 }
 
+// A 64-bit integer as a double in two FP64 additions: each half becomes the low bits of a
+// double's mantissa (at 2^52 and 2^84), whose offsets are then taken out.
+__device__ __forceinline__ double to_double(long long v) {
+    const double lo = __hiloint2double(0x43300000, (int)v);                                   // 2^52 + low
+    const double hi = __hiloint2double(0x45300000, (int)((unsigned)(v >> 32) ^ 0x80000000u)); // 2^84 + (high + 2^31) 2^32
+    return (hi - (0x1.0p84 + 0x1.0p63 + 0x1.0p52)) + lo;
+}
+
 // K4a, one thread per edge: in the FP32 build its current from the sums of its triangles;
 // on free edges r = D_curl^T star_mu^-1 B^{n+1/2} - J^{n+1/2} and the DGL auxiliary flux
 // D += dt r.  The first blocks record probes and ports (record.h).
@@ -119,6 +127,8 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
 // diagnostics compare); in both builds the charge removed at walls is summed since the
 // Gauss-law reference.
 //
+// FP64 instructions take 16 cycles of an SM each (49% of its time on the 200k-triangle mesh
+// with the integer and dt converted by the compiler's rules): r and D need five.
 // Bound by the sectors it gathers from triangles that lie anywhere in memory: two an edge
 // and six a node, of 32 bytes each (with B, star_mu^-1 and the sums in arrays of their own
 // it was six an edge, and eight surrogate instances' 64 steps took 2956 us instead of 2676).
@@ -164,13 +174,12 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
     }
     chain_wait();
     if (e < a.N1) {
-        double r = 0;
+        double h[2] = {0.0, 0.0};
         long long J = 0;
 #pragma unroll
         for (int q = 0; q < 2; q++) {
             if (fs[q] == 0) continue;
             const int fk = abs(fs[q]) - 1, f = fk >> 2;
-            double hf;
             if constexpr (P::fixed) {
                 const longlong2 *F = reinterpret_cast<const longlong2 *>(a.face + f);
                 const longlong2 d = F[0], ah = F[1];
@@ -178,19 +187,21 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
                 if ((fk & 3) != 1) A += d.x << LAM_BITS;             // edge 2
                 if ((fk & 3) == 0) A += d.y << LAM_BITS;             // edge 0
                 J += fs[q] > 0 ? A : -A;
-                hf = __longlong_as_double(ah.y);
+                h[q] = __longlong_as_double(ah.y);
             } else {
-                hf = mu[q] * a.B[f];
+                h[q] = mu[q] * a.B[f];
             }
-            r += fs[q] > 0 ? hf : -hf;
+            if (fs[q] < 0) h[q] = -h[q];
         }
         if constexpr (P::fixed) a.J[e] = (unsigned long long)J;
         if (i >= 0) {
-            double Jp;
-            if constexpr (P::fixed) Jp = (double)J * a.j_scale;
-            else Jp = a.J[e] * a.j_scale;
-            r -= Jp;
-            a.D[e] += (double)a.dt * r;
+            double r = h[0] + h[1];
+            if constexpr (P::fixed) {
+                if (J != 0) r -= to_double(J) * a.j_scale;   // no beam over most of a mesh
+            } else {
+                r -= a.J[e] * a.j_scale;
+            }
+            a.D[e] += a.dt64 * r;
             a.r[i] = (R)r;
         }
     }
@@ -214,9 +225,10 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
 
 // K4b, sliced ELL SpMV over free edges: E_e += dt (M r)_i (in a lossy layer
 // E_e <- a_e E_e + b_e dt (M r)_i, a = (1 - s)/(1 + s), b = 1/(1 + s), s = sigma dt/(2 eps0)).  A warp owns a slice of 32 rows
-// stored column-major, so each step of the row loop reads 32 consecutive values.
+// stored column-major, so each step of the row loop reads 32 consecutive values.  FP32: at
+// most 32 registers, so that 300k rows are one wave (40 took 1% of a step more).
 template <class P, bool LOSS>
-__global__ void __launch_bounds__(512) k_field_spmv(const __grid_constant__ FieldArgs<P> a) {
+__global__ void __launch_bounds__(512, sizeof(typename P::R) == 4 ? 4 : 1) k_field_spmv(const __grid_constant__ FieldArgs<P> a) {
     using R = typename P::R;
     int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t slice = row >> 5;

@@ -245,17 +245,28 @@ void note_launches(long long k);
 long long launches_this_thread();
 #define PIC_LAUNCHED() ::pic::note_launches(1)
 
-// Launch of a kernel of a dependent chain: its blocks may take their places while the
-// kernel before it drains, and wait there (griddepcontrol.wait, the kernel's first
-// statement) until that one has completed and its writes are visible.  The kernel lets its
-// own successor in the same way right after its wait (griddepcontrol.launch_dependents),
-// so that whatever a kernel has waited for has completed before its successor starts.
+// Launch of a kernel of a dependent chain: its blocks may take their places before the
+// kernel ahead of it has completed and its writes are visible, and wait for that
+// (griddepcontrol.wait, in chain_wait, ahead of which a kernel only reads what no kernel of
+// the chain writes).
+//
+// When the blocks of the kernel behind may come is the kernel ahead's choice, made after its
+// own wait, so that whatever a kernel has waited for has completed before its successor
+// starts.  A small grid (at most CHAIN_EARLY threads) leaves most SMs idle and lets them come
+// at once; a large one as its own blocks finish, because blocks that wait hold places and
+// registers that working ones could use.  Measured, at once / as blocks finish / by this
+// rule: 200 FP64 steps on 2000 triangles with 10,000 particles 1971 / 2075 /
+// 2001 us, 8 of 1M FP64 particles on 199k triangles 3267 / 2827 / 2842 us, 64 of eight
+// surrogate instances 2600 / 2327 / 2283 us, 16M particles 290 / 285 / 284 us a step.
+//
 // chain = false: an ordinary launch, for the first kernel of a call and for one that
 // follows an event wait (what it depends on is then not a kernel of this stream).
+constexpr unsigned CHAIN_EARLY = 32768;
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (gridDim.x * gridDim.y * blockDim.x <= CHAIN_EARLY)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 template <class... Params, class... Args>
@@ -459,6 +470,7 @@ struct FieldArgs {
     const typename P::R *ell_val;
     int64_t N1, N2, nf;
     typename P::R dt;
+    double dt64;                // dt as the fields see it: (double)dt
     double j_scale;             // physical J = J_acc * j_scale
     // FP32 build: Q^{n+1} = Q^n - D_div J / 2^22 - Q_absorbed per node (exact)
     const int32_t *face_ptr;    // N0 + 1: node -> incident triangles

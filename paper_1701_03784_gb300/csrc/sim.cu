@@ -452,6 +452,7 @@ struct SimImpl final : SimBase {
         a.N2 = m->N2;
         a.nf = nf;
         a.dt = (R)dt;
+        a.dt64 = (double)a.dt;
         a.j_scale = j_scale();
         a.free_of_edge = free_of_edge;
         a.face = face;
