@@ -59,7 +59,8 @@ struct MlpTc {
     long long wmember = 0, bmember = 0;                     // elements per member
     uint16_t *w = nullptr;                                  // E * wmember BF16
     float *b = nullptr;                                     // E * bmember
-    unsigned int *err = nullptr;                            // bounded-wait timeouts
+    unsigned int *err = nullptr;                            // bounded-wait timeouts: a word of
+                                                            // mapped host memory, zero between calls
     long long wait_polls = 1LL << 22;                       // polls of a pipeline wait
     bool ok = false;
 };
@@ -499,7 +500,8 @@ void launch_deposit_q(const TriRec<typename P::R> *rec, Particles<P> p, int64_t 
                       int64_t count, const int64_t *n_slots, typename P::Acc *Q, cudaStream_t s);
 
 struct SortScratch {
-    int32_t *cnt = nullptr;      // N2 + 1: counts, then write cursors
+    int32_t *cnt = nullptr;      // N2: counts, zero between re-sorts
+    int32_t *cursor = nullptr;   // N2: write cursors
     int32_t *blk = nullptr;      // scan chunk sums
     int64_t *n_old = nullptr;    // slot count before the sort
 };
@@ -507,7 +509,7 @@ struct SortScratch {
 // slot count to n_slots[0] and n_slots[1] (device)
 template <class P>
 void launch_resort(Particles<P> src, Particles<P> dst, int64_t *n_slots, int64_t n_bound,
-                   int64_t N2, const SortScratch &sc, cudaStream_t s);
+                   int64_t N2, const SortScratch &sc, bool chain, cudaStream_t s);
 
 // diagnostics, FP64 reductions on the device
 struct DiagDev {

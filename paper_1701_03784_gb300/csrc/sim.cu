@@ -393,9 +393,10 @@ struct SimImpl final : SimBase {
         PIC_CUDA_TRY(cudaMemset(d_n, 0, 2 * sizeof(int64_t)));
         PIC_CUDA_TRY(cudaMemset(counters, 0, sizeof(unsigned long long) * CNT_N));
         // sort scratch
-        if ((st = dalloc(sc.cnt, mesh.N2 + 1)) || (st = dalloc(sc.blk, mesh.N2 / 2048 + 2)) ||
-            (st = dalloc(sc.n_old, 1)))
+        if ((st = dalloc(sc.cnt, mesh.N2)) || (st = dalloc(sc.cursor, mesh.N2)) ||
+            (st = dalloc(sc.blk, mesh.N2 / 2048 + 2)) || (st = dalloc(sc.n_old, 1)))
             return st;
+        PIC_CUDA_TRY(cudaMemset(sc.cnt, 0, sizeof(int32_t) * mesh.N2));
         // diagnostics: node -> edge incidence (D_div rows), star_eps
         std::vector<int64_t> nptr(mesh.N0 + 1, 0);
         for (int64_t e = 0; e < mesh.N1; e++) {
@@ -801,8 +802,8 @@ struct SimImpl final : SimBase {
         return PIC_OK;
     }
 
-    pic_status resort(cudaStream_t s) {
-        launch_resort<P>(parts[cur], parts[1 - cur], d_n, n_bound, m->N2, sc, s);
+    pic_status resort(bool chain, cudaStream_t s) {
+        launch_resort<P>(parts[cur], parts[1 - cur], d_n, n_bound, m->N2, sc, chain, s);
         cur = 1 - cur;
         since_sort = 0;
         return PIC_OK;
@@ -903,7 +904,7 @@ struct SimImpl final : SimBase {
             PIC_CUDA_TRY(cudaMemcpyAsync(counters + CNT_NEXT_PID, &np, sizeof np, cudaMemcpyHostToDevice, s));
         }
         n_injected += n;
-        resort(s);
+        resort(false, s);
         PIC_CUDA_TRY(cudaGetLastError());
         PIC_CUDA_TRY(cudaStreamSynchronize(s));
         dgl_dirty = true;
@@ -1124,7 +1125,7 @@ struct SimImpl final : SimBase {
         launch_field_e<P>(fa, probes_on ? probe : ProbeArgs<P>{}, ports_on ? port : PortArgs<P>{}, s);
         qcur = 1 - qcur;
         n_steps++;
-        if (sort_interval > 0 && ++since_sort >= sort_interval) resort(s);
+        if (sort_interval > 0 && ++since_sort >= sort_interval) resort(true, s);
     }
 
     pic_status step_direct(int64_t n, cudaStream_t s) {
