@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(NTH, MIN_BLOCKS) k_mlp_tc(MlpTc tc, const floa
             }
         }
     }
-    if (!ok) atomicAdd(tc.err, 1u);
+    if (!ok) atomicAdd_system(tc.err, 1u);
     fence_before();
     __syncthreads();
     fence_after();
@@ -641,10 +641,15 @@ pic_status mlp_tc_forward(const MlpTc &tc, const float *X, float *Y, int64_t n, 
         return PIC_ERR_ARG;
     }
     const int smem = (int)sizeof(PingSmem) + 1024;
-    PIC_CUDA_TRY(cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    PIC_CUDA_TRY(cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared));
-    PIC_CUDA_TRY(cudaMemsetAsync(tc.err, 0, sizeof(unsigned int), s));
+    static bool attr[64] = {};   // the shared-memory opt-in, once per device
+    int dev = 0;
+    PIC_CUDA_TRY(cudaGetDevice(&dev));
+    if (!attr[dev & 63]) {
+        PIC_CUDA_TRY(cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        PIC_CUDA_TRY(cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                          (int)cudaSharedmemCarveoutMaxShared));
+        attr[dev & 63] = true;
+    }
     // grid: members along x, pairs of tiles along y (at most 65535 pairs per launch)
     const long long pairs = (n + NTILE * TM - 1) / (NTILE * TM);
     for (long long p0 = 0; p0 < pairs; p0 += 65535) {
@@ -654,9 +659,9 @@ pic_status mlp_tc_forward(const MlpTc &tc, const float *X, float *Y, int64_t n, 
         PIC_LAUNCHED();
     }
     PIC_CUDA_TRY(cudaGetLastError());
-    unsigned int err = 0;
-    PIC_CUDA_TRY(cudaMemcpyAsync(&err, tc.err, sizeof(err), cudaMemcpyDeviceToHost, s));
     PIC_CUDA_TRY(cudaStreamSynchronize(s));
+    const unsigned int err = *static_cast<volatile unsigned int *>(tc.err);
+    *tc.err = 0;
     if (err) {
         set_error("pic_mlp_forward: %u tensor-core waits timed out", err);
         return PIC_ERR_TIMEOUT;

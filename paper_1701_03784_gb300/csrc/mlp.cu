@@ -164,6 +164,7 @@ struct MlpImpl {
     ~MlpImpl() {
         cudaSetDevice(device);
         cudaDeviceSynchronize();
+        if (tc.err) cudaFreeHost(tc.err);
         for (void *p : allocs) {
             if (al.free) al.free(p, al.ctx);
             else cudaFree(p);
@@ -246,7 +247,6 @@ struct MlpImpl {
             }
             carve.want(tc.w, E * tc.wmember);
             carve.want(tc.b, E * tc.bmember);
-            carve.want(tc.err, 1);
             const long long mp = (std::max(max_batch, maxw) + 127) / 128 * 128;
             carve.want(tsa, (long long)E * mp * 256);
             carve.want(tsb, (long long)E * 256 * 256);
@@ -277,6 +277,11 @@ struct MlpImpl {
         for (const auto &x : carve.at) *x.first = base + x.second;
         PIC_CUDA_TRY(cudaMemset(base, 0, cleared));
         if (terr) PIC_CUDA_TRY(cudaMemset(terr, 0, sizeof(unsigned int)));
+        if (tc.ok) {
+            // read by the host once the stream is done, without a copy
+            PIC_CUDA_TRY(cudaHostAlloc(&tc.err, sizeof(unsigned int), cudaHostAllocMapped | cudaHostAllocPortable));
+            *tc.err = 0;
+        }
         return PIC_OK;
     }
 
