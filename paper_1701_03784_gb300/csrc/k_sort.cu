@@ -57,6 +57,23 @@ __device__ __forceinline__ int ht_find(const SortTable &h, int t) {
     return -1;
 }
 
+// A block puts its particles of a triangle down part by part: particles that stay together
+// reach the next triangle together, and the particle kernel takes the sums of a warp's
+// triangles one after another (a launch on 16M takes 213 us right after a re-sort and 247 us
+// eight steps on).  Parts 1, 4, 16, 64: the launches of 16 steps 244.7, 239.0, 235.4, 240.1 us
+// on average, a step with its share of the re-sort 282.5, 279.6, 278.8, 287.3 us (16M), 105.1,
+// 104.6, 106.6, 111.3 us (5M spread over 50k triangles).
+// (The FP64 kernel adds particle by particle: no parts.)
+template <class P>
+constexpr int PARTS = P::fixed ? 4 : 1;
+// which of the triangle's four halved copies holds the point: a corner's or the middle one
+template <class P>
+__device__ __forceinline__ int part_of(typename P::Lam l0, typename P::Lam l1) {
+    if constexpr (PARTS<P> == 1) return 0;
+    constexpr int HALF = LAM_ONE / 2;
+    return l0 >= HALF ? 0 : l1 >= HALF ? 1 : l0 + l1 <= HALF ? 2 : 3;
+}
+
 __device__ __forceinline__ void ht_clear(SortTable &h) {
     for (int e = threadIdx.x; e < HT; e += blockDim.x) {
         h.key[e] = -1;
@@ -185,31 +202,34 @@ __global__ void __launch_bounds__(256) k_scatter(Particles<P> src, Particles<P> 
             pid[k] = __ldcs(src.pid + i);
         }
     }
+    int key[SORT_PER];   // triangle and part of it
+#pragma unroll
+    for (int k = 0; k < SORT_PER; k++) key[k] = t[k] >= 0 ? t[k] * PARTS<P> + part_of<P>(l0[k], l1[k]) : -1;
     ht_clear(h);
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < SORT_PER; k++) {
-        const unsigned grp = __match_any_sync(full, t[k]);
-        if (t[k] >= 0 && lane == __ffs(grp) - 1) {
-            const int e = ht_insert(h, t[k]);
+        const unsigned grp = __match_any_sync(full, key[k]);
+        if (key[k] >= 0 && lane == __ffs(grp) - 1) {
+            const int e = ht_insert(h, key[k]);
             if (e >= 0) atomicAdd(&h.cnt[e], __popc(grp));
         }
     }
     __syncthreads();
-    // one range of the sorted order per triangle of the chunk
+    // one range of the sorted order per triangle and part of the chunk
     for (int e = threadIdx.x; e < HT; e += 256) {
-        const int key = h.key[e];
-        if (key >= 0) h.base[e] = atomicAdd(cursor + key, h.cnt[e]);
+        const int q = h.key[e];
+        if (q >= 0) h.base[e] = atomicAdd(cursor + q / PARTS<P>, h.cnt[e]);
         h.cnt[e] = 0;
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < SORT_PER; k++) {
-        const unsigned grp = __match_any_sync(full, t[k]);
+        const unsigned grp = __match_any_sync(full, key[k]);
         const int leader = __ffs(grp) - 1;
         int pos = 0;
-        if (t[k] >= 0 && lane == leader) {
-            const int e = ht_find(h, t[k]);
+        if (key[k] >= 0 && lane == leader) {
+            const int e = ht_find(h, key[k]);
             pos = e >= 0 ? h.base[e] + atomicAdd(&h.cnt[e], __popc(grp))
                          : atomicAdd(cursor + t[k], __popc(grp));
         }
