@@ -239,7 +239,7 @@ struct MlpImpl {
                 tc.k[l] = sz[l];
                 tc.n[l] = sz[l + 1];
                 tc.kp[l] = (sz[l] + 15) / 16 * 16;
-                tc.np[l] = (sz[l + 1] + 15) / 16 * 16;
+                tc.np[l] = (sz[l + 1] + 31) / 32 * 32;   // half in each CTA of a pair
                 tc.woff[l] = tc.wmember;
                 tc.wmember += (long long)tc.kp[l] * tc.np[l];
                 tc.boff[l] = tc.bmember;

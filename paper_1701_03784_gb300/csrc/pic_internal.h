@@ -47,14 +47,14 @@ struct Allocator {
 Allocator current_allocator();
 
 // Tensor-core inference state of a surrogate network (k_mlp_tc.cu): BF16 weights of every
-// member and layer, zero-padded to multiples of 16 and stored in the tensor core's
-// no-swizzle K-major layout (8 x 8 core matrices, K-adjacent ones contiguous), and FP32
-// biases.  Usable when every layer width is at most 256.
+// member and layer, zero-padded (inputs to multiples of 16, outputs to multiples of 32: a pair
+// of SMs takes half each) and stored in the tensor core's no-swizzle K-major layout (8 x 8 core
+// matrices, K-adjacent ones contiguous), and FP32 biases.  Usable when every layer width is at most 256.
 constexpr int MLP_MAX_LAYERS = 16;
 struct MlpTc {
     int E = 0, L = 0;
     int k[MLP_MAX_LAYERS] = {}, n[MLP_MAX_LAYERS] = {};    // widths: in, out
-    int kp[MLP_MAX_LAYERS] = {}, np[MLP_MAX_LAYERS] = {};  // padded to multiples of 16
+    int kp[MLP_MAX_LAYERS] = {}, np[MLP_MAX_LAYERS] = {};  // padded to 16 and 32
     long long woff[MLP_MAX_LAYERS] = {}, boff[MLP_MAX_LAYERS] = {};
     long long wmember = 0, bmember = 0;                     // elements per member
     uint16_t *w = nullptr;                                  // E * wmember BF16
