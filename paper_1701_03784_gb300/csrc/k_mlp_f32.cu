@@ -10,20 +10,6 @@ namespace pic {
 
 namespace {
 
-// ---- asynchronous copies global -> shared ----------------------------------------------
-// 16 or 4 bytes, of which the first `bytes` are read and the rest become zeros
-__device__ __forceinline__ void cp16(float *dst, const float *src, int bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                     (unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp4(float *dst, const float *src, int bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                     (unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // =========================================================================================
 // Layer products
 // =========================================================================================
@@ -43,7 +29,7 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 // (4 x 4 elements a thread, the tile split over the warps) ask half the L2 bandwidth a
 // flop and take over once they fill the SMs twice (mlp_jobs).
 //
-// Measured, a training step of 5 x 6 -> 4 x 256 -> 33 at batch 128: 86 us in 11 launches
+// Measured, a training step of 5 x 6 -> 4 x 256 -> 33 at batch 128: 84 us in 11 launches
 // (335 us in 31 with 16 x 16 tiles of one element a thread and separate bias, activation,
 // column-sum and Adam kernels); batch 256: 129 us; 4 x 64 units: 44 us, which is what the
 // host takes to enqueue 11 launches.

@@ -362,8 +362,62 @@ struct MlpImpl {
     // parameters' step in the place of the gradients' storing.  The weight gradients of a
     // layer go with the next input gradient, which reads other weights.
     void fused_step(int rows, float *loss_out, const AdamArgs *adam, cudaStream_t s) {
+        bool whole = false;
+        if (f32.ok) {
+            MlpChain c{};
+            c.E = E;
+            c.L = L;
+            c.rows = rows;
+            c.batch = max_batch;
+            c.P = P;
+            c.params = params;
+            c.T = Tb;
+            for (int l = 0; l <= L; l++) c.sz[l] = sz[l];
+            for (int l = 0; l < L; l++) {
+                c.woff[l] = woff[l];
+                c.boff[l] = boff[l];
+                c.act[l] = act[l];
+                c.pre[l] = pre[l];
+            }
+            c.scale = 2.f / (float)((long long)rows * sz[L]);
+            c.loss = loss_out;
+            whole = mlp_chain(c, true, s);
+        }
         const long long sg = (long long)max_batch * maxw;
         const auto sa = [&](int l) { return (long long)max_batch * sz[l]; };
+        const auto dw = [&](int l) {
+            MlpJob j{};
+            j.kind = MLP_DW;
+            j.M = j.lda = sz[l + 1];
+            j.N = j.ldb = j.ldc = sz[l];
+            j.K = rows;
+            j.A = whole ? pre[l] : gbuf[l % 3];
+            j.sA = whole ? sa(l + 1) : sg;
+            j.B = act[l];
+            j.sB = sa(l);
+            j.sC = P;
+            if (adam) {
+                j.epi = MLP_EPI_ADAM;
+                j.adam = *adam;
+                j.C = params + woff[l];
+                j.am = am + woff[l];
+                j.av = av + woff[l];
+                j.db = params + boff[l];
+                j.dbm = am + boff[l];
+                j.dbv = av + boff[l];
+            } else {
+                j.epi = MLP_EPI_STORE;
+                j.C = grads + woff[l];
+                j.db = grads + boff[l];
+            }
+            return j;
+        };
+        if (whole) {   // pre: the gradients by the layers' sums
+            MlpJobs jobs;
+            for (int l = L - 1; l >= 0; l--) jobs.job[jobs.n++] = dw(l);
+            mlp_jobs(jobs, E, true, s);
+            return;
+        }
         for (int l = 0; l < L; l++) {
             MlpJobs jobs;
             const bool last = l == L - 1;
@@ -395,33 +449,6 @@ struct MlpImpl {
             j.C = gbuf[(l - 1) % 3];
             j.Z = pre[l - 1];
             j.sZ = sa(l);
-            return j;
-        };
-        const auto dw = [&](int l) {
-            MlpJob j{};
-            j.kind = MLP_DW;
-            j.M = j.lda = sz[l + 1];
-            j.N = j.ldb = j.ldc = sz[l];
-            j.K = rows;
-            j.A = gbuf[l % 3];
-            j.sA = sg;
-            j.B = act[l];
-            j.sB = sa(l);
-            j.sC = P;
-            if (adam) {
-                j.epi = MLP_EPI_ADAM;
-                j.adam = *adam;
-                j.C = params + woff[l];
-                j.am = am + woff[l];
-                j.av = av + woff[l];
-                j.db = params + boff[l];
-                j.dbm = am + boff[l];
-                j.dbv = av + boff[l];
-            } else {
-                j.epi = MLP_EPI_STORE;
-                j.C = grads + woff[l];
-                j.db = grads + boff[l];
-            }
             return j;
         };
         for (int l = L - 1; l >= 1; l--) {

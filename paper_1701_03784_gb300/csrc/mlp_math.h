@@ -1,4 +1,4 @@
-// Elementwise arithmetic of the surrogate networks, shared by the FP32 kernels.
+// Elementwise arithmetic and copies of the surrogate networks, shared by the FP32 kernels.
 #pragma once
 
 #include "pic_internal.h"
@@ -23,5 +23,19 @@ __device__ __forceinline__ void adam_step(const AdamArgs &a, float gi, float &p,
     v = vi;
     p -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
 }
+
+// ---- asynchronous copies global -> shared ----------------------------------------------
+// 16 or 4 bytes, of which the first `bytes` are read and the rest become zeros
+__device__ __forceinline__ void cp16(float *dst, const float *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp4(float *dst, const float *src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 }  // namespace pic

@@ -116,7 +116,7 @@ struct MlpJob {
     float *loss;
     AdamArgs adam;
 };
-constexpr int MLP_MAX_JOBS = 3;
+constexpr int MLP_MAX_JOBS = MLP_MAX_LAYERS;
 struct MlpJobs {
     MlpJob job[MLP_MAX_JOBS];   // in the order that the blocks take them
     int blocks[MLP_MAX_JOBS];
@@ -124,6 +124,22 @@ struct MlpJobs {
 };
 // the jobs in one launch (their results must not depend on each other)
 void mlp_jobs(MlpJobs &jobs, int E, bool chain, cudaStream_t s);
+
+// A batch's forward products, loss and gradients by the layers' sums (k_mlp_chain.cu): every
+// width at most 256.
+struct MlpChain {
+    int E, L, rows;
+    int sz[MLP_MAX_LAYERS + 1];
+    long long batch, P;                                    // rows the arrays hold; member stride
+    const float *params, *T;                               // parameters; targets (batch x outputs)
+    long long woff[MLP_MAX_LAYERS], boff[MLP_MAX_LAYERS];
+    float *act[MLP_MAX_LAYERS];                            // layer l's inputs; act[0] is read
+    float *pre[MLP_MAX_LAYERS];                            // gradients by layer l's sums, on return
+    float scale;                                           // of the gradient by the outputs
+    float *loss;                                           // per member, added to; or null
+};
+// false: not for this many rows, nothing launched
+bool mlp_chain(const MlpChain &a, bool chain, cudaStream_t s);
 
 // Parameters as the whole-network kernel reads them: per member and layer the weights
 // k-major (kp x np: kp the inputs up to a multiple of 16, np by mlp_f32_shape) and np biases.
