@@ -14,10 +14,11 @@
 // What bounds it: of a product's 12k cycles at 24 rows and 256 x 256, the product 5.7k
 // (shared-memory reads: ten 16-byte loads a lane for 96 FMAs, 5.1k), the copies of 64 KB of weights a
 // CTA 2.4k, sums, activation and exchange 2.8k, the barrier 1k.  A step of five members of
-// 6 -> 4 x 256 -> 33 at batch 128 takes 71 us in 3 launches (84 us in 11 layer by layer), 50 of
-// them here.  Results written to memory ahead of the barrier's arrival: 72 us; eight warps
-// with twice the rows a thread: 77 us; 8 columns a thread and two warps that bring the
-// weights: 86 us.
+// 6 -> 4 x 256 -> 33 at batch 128 takes 67 us in 3 launches (84 us in 11 layer by layer), 48 of
+// them here.  Unrolled twice over k, with spills: 2 us more; results written to memory ahead
+// of the barrier's arrival: 3 more; eight warps with twice the rows a thread: 7 more; sixteen
+// slices of k, 10 rows a thread: as fast, but narrow layers slower by a tenth; 8 columns a
+// thread and two warps that bring the weights: 16 more.
 #include "mlp_math.h"
 #include "pic_internal.h"
 
@@ -93,7 +94,7 @@ __device__ __forceinline__ float4 at4(const float *p) { return *reinterpret_cast
 template <int RT, bool FWD>
 __device__ __forceinline__ void partial(const float *in, const float *w, int quads, int g, int cg, float *out) {
     float acc[RT][4] = {};
-#pragma unroll 2
+#pragma unroll 1
     for (int q = 0; q < quads; q++) {
         float4 b[4];
 #pragma unroll
@@ -302,8 +303,8 @@ void launch(const MlpChain &a, bool chain, cudaStream_t s) {
 
 // The fewest rows a CTA with which one round of clusters does: more rounds, or layers of which
 // the product's columns fill little, go faster layer by layer (us a step, here and there:
-// 5 members of 4 x 256, batch 128: 71 / 84, 512: 231 / 210; of 4 x 64, batch 128: 35 / 44, 1024:
-// 179 / 135; 8 of 5 x 100, batch 64: 43 / 58, 256: 141 / 98; one of 4 x 256, batch 700: 71 / 112).
+// 5 members of 4 x 256, batch 128: 67 / 84, 512: 231 / 210; of 4 x 64, batch 128: 33 / 44, 1024:
+// 179 / 135; 8 of 5 x 100, batch 64: 42 / 58, 256: 141 / 98; one of 4 x 256, batch 700: 69 / 112).
 bool mlp_chain(const MlpChain &a, bool chain, cudaStream_t s) {
     const auto fits = [&](int rt, int cap) { return a.E * (((long long)a.rows + RG * rt - 1) / (RG * rt)) <= cap; };
     if (fits(2, slots<2>())) launch<2>(a, chain, s);

@@ -29,10 +29,10 @@ namespace {
 // (4 x 4 elements a thread, the tile split over the warps) ask half the L2 bandwidth a
 // flop and take over once they fill the SMs twice (mlp_jobs).
 //
-// Measured, a training step of 5 x 6 -> 4 x 256 -> 33 at batch 128: 84 us in 11 launches
-// (335 us in 31 with 16 x 16 tiles of one element a thread and separate bias, activation,
-// column-sum and Adam kernels); batch 256: 129 us; 4 x 64 units: 44 us, which is what the
-// host takes to enqueue 11 launches.
+// Measured, a training step of 5 x 6 -> 4 x 256 -> 33 at batch 128: 84 us in 11 launches (335 us
+// in 31 with 16 x 16 tiles of one element a thread and separate bias, activation, column-sum
+// and Adam kernels; 67 us with all but the weight gradients in one kernel, k_mlp_chain.cu);
+// batch 256: 128 us.
 constexpr int BK = 32;
 
 template <int T>
@@ -558,7 +558,10 @@ void mlp_jobs(MlpJobs &jobs, int E, bool chain, cudaStream_t s) {
     long long big = 0;
     for (int j = 0; j < jobs.n; j++)
         big += (long long)((jobs.job[j].M + 63) / 64) * ((jobs.job[j].N + 63) / 64) * E;
-    const int T = big >= 2 * sm_count() ? 64 : 32;
+    // one block an SM and a half are enough behind nothing that waits for the last of them: all
+    // weight gradients in one launch (a step of 5 x 4 x 256 at batch 128 / 64 / 16 with 280 blocks
+    // of 64 x 64: 67.4 / 55.3 / 46.7 us, 32 x 32: 69.7 / 57.2 / 48.1; with 160 blocks 46.9 and 42.2)
+    const int T = 2 * big >= (jobs.n > 2 ? 3 : 4) * sm_count() ? 64 : 32;
     long long blocks = 0;
     for (int j = 0; j < jobs.n; j++) {
         jobs.blocks[j] = (int)((long long)((jobs.job[j].M + T - 1) / T) * ((jobs.job[j].N + T - 1) / T) * E);
