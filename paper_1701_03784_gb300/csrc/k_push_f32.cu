@@ -449,25 +449,26 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         float sP = fP * rcp(fP - leP), sQ = fQ * rcp(fQ - leQ);
         sP = xP ? sP : 2.f;
         sQ = xQ ? sQ : 2.f;
-        const bool atP = sP <= sQ;
+        const bool atP = j == 1 ? sP < sQ : sP <= sQ;   // the lower edge where both are reached at once
         sx = atP ? sP : sQ;
         const float cR = fmaxf(__fmul_rn(sx, dR), 0.f);
         const float cS = fmaxf(__fmaf_rn(sx, atP ? dQ : dP, atP ? fQ : fP), 0.f);
-        const int qS = edge_point(cS, cR), qR = LAM_ONE - qS;
-        ea = atP ? qS : qR;
-        eb = atP ? qR : qS;
-        // staying: R takes what rounding leaves, a deficit goes to the larger of P and Q
-        int iP = f2fix(fmaxf(leP, 0.f)), iQ = f2fix(fmaxf(leQ, 0.f));
-        const int iR = LAM_ONE - iP - iQ, neg = min(iR, 0);
-        const bool bigP = iP >= iQ;
-        iP += bigP ? neg : 0;
-        iQ += bigP ? 0 : neg;
-        const int eP = leaves ? (atP ? 0 : qS) : iP;
-        const int eQ = leaves ? (atP ? qS : 0) : iQ;
-        const int eR = leaves ? qR : iR - neg;
-        // Eq. current from (0, P, Q) at nodes (j, j+1, j+2)
+        ea = edge_point(atP ? cS : cR, atP ? cR : cS);
+        eb = LAM_ONE - ea;
+        const int qS = atP ? ea : eb, qR = atP ? eb : ea;
+        const int eP = leaves ? (atP ? 0 : qS) : f2fix(fmaxf(leP, 0.f));
+        const int eQ = leaves ? (atP ? qS : 0) : f2fix(fmaxf(leQ, 0.f));
+        const int eR = leaves ? qR : f2fix(fmaxf(dR, 0.f));
         l0 = sel3(j, eR, eQ, eP);
         l1 = sel3(j, eP, eR, eQ);
+        // staying, node 2 takes what rounding leaves, a deficit goes to the larger of the others
+        // (as segment_end: rounding the other way round would move a particle beside the axis
+        // by its distance from it)
+        const int neg = min(LAM_ONE - l0 - l1, 0);
+        const bool big0 = l0 >= l1;
+        l0 += big0 ? neg : 0;
+        l1 += big0 ? 0 : neg;
+        // Eq. current from (0, P, Q) at nodes (j, j+1, j+2)
         const int t0 = sel3(j, 0, Q, P), t1 = sel3(j, P, 0, Q);
         add_current(a, t, (long long)(LAM_ONE - t0 - t1) * l0 - (long long)t0 * (LAM_ONE - l0 - l1), t0 - l0,
                     t1 - l1);
