@@ -226,10 +226,12 @@ inline void edge_tail_head(const int32_t *n3, int k, int *a, int *b) {
     if (n3[i] < n3[j]) { *a = i; *b = j; } else { *a = j; *b = i; }
 }
 
-// run f(begin, end) over [0, n) on the host's cores
+// run f(begin, end) over [0, n) on the host's cores, at least `grain` items a thread: a
+// thread takes some 30 us to start, so light loops ask for thousands
 template <class F>
-void parallel_for(int64_t n, F &&f) {
+void parallel_for(int64_t n, F &&f, int64_t grain = 1) {
     unsigned nt = std::max(1u, std::min(64u, std::thread::hardware_concurrency()));
+    nt = (unsigned)std::max<int64_t>(1, std::min<int64_t>(nt, n / grain));
     if (n < 4096 || nt == 1) {
         f((int64_t)0, n);
         return;

@@ -272,6 +272,7 @@ struct SimImpl final : SimBase {
         nf = (int64_t)mesh.free_edges.size();
         PIC_CUDA_TRY(cudaGetDevice(&device));
         pic_status st;
+        constexpr int64_t GRAIN = 16384;   // some 10 ns an item in the loops below
         // triangle records
         std::vector<TriRec<R>> hr(mesh.N2);
         parallel_for(mesh.N2, [&](int64_t t_a, int64_t t_b) {
@@ -304,7 +305,7 @@ struct SimImpl final : SimBase {
                 x.entry = entry;
                 x.inv_area = (R)(1.0 / mesh.area[t]);
             }
-        });
+        }, GRAIN);
         if ((st = upload(rec, hr)) != PIC_OK) return st;
         std::vector<R> hmu(mesh.mu_inv.begin(), mesh.mu_inv.end());
         if ((st = upload(mu_inv, hmu)) != PIC_OK) return st;
@@ -317,7 +318,7 @@ struct SimImpl final : SimBase {
                     const int64_t q2 = 2 * e + (mesh.edge_face[2 * e] == f ? 0 : 1);
                     hef[q2] = (int32_t)(4 * f + k + 1) * mesh.edge_face_sign[q2];
                 }
-        });
+        }, GRAIN);
         if ((st = upload(free_of_edge, mesh.free_of_edge)) != PIC_OK) return st;
         if constexpr (P::fixed) {
             // the triangles of each node, with the node's place in them
@@ -352,7 +353,7 @@ struct SimImpl final : SimBase {
                     hval[hoff[sl] + 32 * k + lane] = (R)mesh.M_val[q2];
                 }
             }
-        });
+        }, GRAIN);
         if ((st = upload(ell_off, hoff)) != PIC_OK) return st;
         if ((st = upload(ell_col, hcol)) != PIC_OK) return st;
         if ((st = upload(ell_val, hval)) != PIC_OK) return st;
