@@ -25,7 +25,7 @@
 //    the segment to the first edge reached, its currents (added one by one), then the
 //    neighbour (entered through a precomputed local edge index) until the end point,
 //    the axis, a wall or the walk cap.  The remainder (< 32) is walked at the end.
-// What bounds it: the issue rate (about 410 warp instructions per 32 particles, issued in
+// What bounds it: the issue rate (about 420 warp instructions per 32 particles, issued in
 // two cycles of three) and the per-triangle sums, which the hardware takes one member mask
 // after another.  16M particles, 199k triangles, mean of the steps between re-sorts: 242 us
 // = 3.2 TB/s of the 48 B a particle that have to move (287 us with the walk in the
