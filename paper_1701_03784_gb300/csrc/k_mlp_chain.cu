@@ -18,7 +18,8 @@
 // them here.  Unrolled twice over k, with spills: 2 us more; results written to memory ahead
 // of the barrier's arrival: 3 more; eight warps with twice the rows a thread: 7 more; sixteen
 // slices of k, 10 rows a thread: as fast, but narrow layers slower by a tenth; 8 columns a
-// thread and two warps that bring the weights: 16 more.
+// thread and two warps that bring the weights: 16 more; the warps that have no results to
+// finish bringing the weights meanwhile: 4 more.
 #include "mlp_math.h"
 #include "pic_internal.h"
 
