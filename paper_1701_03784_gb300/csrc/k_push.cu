@@ -253,14 +253,18 @@ __global__ void __launch_bounds__(32 * PW) k_push_f64(const __grid_constant__ Pu
             d0 = uz * gi;
             const double x = rho + xr;
             const double rn2 = fma(x, x, yp * yp);
-            if (rn2 != 0.0) {
-                const double inv = rsqrt(rn2), cs = x * inv, sn = yp * inv;
-                // rn - rho without cancellation
-                d1 = fma(xr, fma(2.0, rho, xr), yp * yp) / fma(rn2, inv, rho);
+            double inv = 0.0;   // 1 / rn, for rn > 0
+            if (rn2 > 0.0) {
+                inv = rsqrt(rn2);
+                const double cs = x * inv, sn = yp * inv;
                 const double nr = cs * ur + sn * up;
                 up = cs * up - sn * ur;
                 ur = nr;
             }
+            // rn - rho without cancellation, on the axis (rn = 0) too; rounding can leave rho
+            // just below zero, and then rn + rho at or below it
+            const double both = fma(rn2, inv, rho);
+            if (__double_as_longlong(both) > 0) d1 = fma(xr, fma(2.0, rho, xr), yp * yp) / both;
             a.p.ur[i] = ur;
             a.p.up[i] = up;
             a.p.uz[i] = uz;
