@@ -35,6 +35,7 @@
 // (nothing in local memory); fixed <-> float conversions use exact magic-number
 // arithmetic instead of the quarter-rate converters.
 #include <algorithm>
+#include <cfloat>
 
 #include "pic_internal.h"
 
@@ -328,14 +329,26 @@ __device__ __forceinline__ void push_particle(const PushArgs<PF32> &a, int i, in
     const float x = rho + xr;
     const float rn2 = x * x + yp * yp;
     const float d0 = uz * gi * a.dt;
-    float d1 = 0.f;
-    if (rn2 >= 1.17549435e-38f) {   // normal: on the axis there is no direction to turn
-        const float rinv = rsq(rn2);
-        d1 = (2.f * rho * xr + xr * xr + yp * yp) * rcp(rn2 * rinv + rho);
-        const float cs = x * rinv, sn = yp * rinv;
+    float d1;
+    const auto turn = [&](float cs, float sn) {
         const float nr = cs * ur + sn * up;
         up = -sn * ur + cs * up;
         ur = nr;
+    };
+    if (rn2 >= FLT_MIN) {
+        const float rinv = rsq(rn2);
+        d1 = (2.f * rho * xr + xr * xr + yp * yp) * rcp(rn2 * rinv + rho);
+        turn(x * rinv, yp * rinv);
+    } else {
+        // on the axis, where there is no direction to turn to, or within 1e-19 of it, where
+        // squares leave the normal range: those of 2^64 times the point are taken
+        const float xs = x * 0x1p64f, ys = yp * 0x1p64f, r2 = xs * xs + ys * ys;
+        d1 = -rho;
+        if (r2 >= FLT_MIN) {
+            const float rinv = rsq(r2);
+            d1 = fmaf(r2 * rinv, 0x1p-64f, -rho);
+            turn(xs * rinv, ys * rinv);
+        }
     }
     __stcs(a.p.ur + i, ur);
     __stcs(a.p.up + i, up);

@@ -40,7 +40,7 @@ def _positions(arrays, tri, lam):
 
 
 @pytest.mark.parametrize("pusher", ["boris", "vay"])
-@pytest.mark.parametrize("precision", ["fp64"])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
 def test_landing_on_the_axis(pic, precision, pusher):
     """Radially inward from rho = |v| dt: rho + v dt is zero or its rounding, and both have to
     end on the axis (FP32: within the 2^-22 of a cell that positions have, a few times; that
@@ -65,3 +65,19 @@ def test_landing_on_the_axis(pic, precision, pusher):
     d = pic.pic_diagnostics(sim)
     assert d["n_absorbed"] == 0
     assert d["dce_nonzero"] == 0 if precision == "fp32" else d["dce_max"] < 1e-12 * n
+
+
+@pytest.mark.parametrize("speed", [1e-3, 1e-18, 1e-20, 1e-28])
+def test_reflection_at_the_axis(pic, speed):
+    """FP32 (whose coordinates on the axis are exact): from the axis across it at any speed
+    (1e-18 and below: the square of the step, 1e-2 of that, is no normal number), u_rho comes
+    out reversed."""
+    n = 100
+    arrays, sim, dt = _sim(pic, "fp32", n)
+    z, zero = np.linspace(0.1, 0.9, n), np.zeros(n)
+    pic.pic_particles_inject(sim, z, zero, np.full(n, -speed), zero, zero, -1.0, 1.0, 1e-15)
+    pic.pic_step(sim, 1)
+    tri, lam, u = _by_pid(pic.pic_particles_get(sim), n)
+    assert np.all(tri >= 0)
+    assert np.abs(u[:, 0] / speed - 1.0).max() < 1e-6 and np.all(u[:, 1:] == 0.0)
+    assert np.abs(_positions(arrays, tri, lam)[:, 1] - speed * dt).max() < 1e-7
