@@ -128,10 +128,10 @@ __device__ __forceinline__ void kick(double &ur, double &up, double &uz, double 
 }
 
 // Walk one ring entry along its straight meridian segment: per triangle the part to the
-// first edge reached (smallest crossing parameter, ties to the lower edge, never the edge
-// just entered), its current, then the neighbour, where the two shared nodes keep their
-// coordinates; until the end point, the axis, a wall or the walk cap.  Returns the edges
-// reached.
+// first edge reached (smallest crossing parameter, between 0 and 1; ties to the lower edge,
+// never the edge just entered), its current, then the neighbour, where the two shared nodes
+// keep their coordinates; until the end point, the axis, a wall or the walk cap.  Returns the
+// edges reached.
 __device__ __forceinline__ unsigned walk(const PushArgs<PF64> &a, int slot, int t, double l0, double l1,
                                          double d0, double d1) {
     double l[3] = {l0, l1, 1.0 - l0 - l1};
@@ -148,11 +148,12 @@ __device__ __forceinline__ unsigned walk(const PushArgs<PF64> &a, int slot, int 
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             e[k] = l[k] + dl[k];
-            if (k == entered || !negative(e[k])) continue;
-            const double w = l[k] - e[k];
-            if (kx < 0 || below(l[k] * wb, lb * w)) {
+            // a coordinate that rounding left below zero and that does not fall is no exit
+            if (k == entered || !negative(e[k]) || !negative(dl[k])) continue;
+            const double b = __double_as_longlong(l[k]) < 0 ? 0.0 : l[k], w = -dl[k];
+            if (kx < 0 || below(b * wb, lb * w)) {
                 kx = k;
-                lb = l[k];
+                lb = b;
                 wb = w;
             }
         }

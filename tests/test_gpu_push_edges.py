@@ -1,5 +1,6 @@
-"""Particles at places that the particle kernels meet rarely.  Force-free, so every particle
-ends at z + v_z dt, |rho + v_rho dt|."""
+"""Particles at places that the particle kernels meet rarely: landing exactly on the axis, and
+coordinates that rounding left just below zero.  Force-free, so every particle ends at
+z + v_z dt, |rho + v_rho dt|."""
 import numpy as np
 import pytest
 
@@ -81,3 +82,64 @@ def test_reflection_at_the_axis(pic, speed):
     assert np.all(tri >= 0)
     assert np.abs(u[:, 0] / speed - 1.0).max() < 1e-6 and np.all(u[:, 1:] == 0.0)
     assert np.abs(_positions(arrays, tri, lam)[:, 1] - speed * dt).max() < 1e-7
+
+
+def _raw_state(pic, sim, precision, tri, l0, l1, u):
+    """One slot per entry, written through the raw layout (pic_particles_raw_set)."""
+    import torch
+    n = len(tri)
+    stride = (n + 31) // 32 * 32
+    real = np.float64 if precision == "fp64" else np.float32
+    lam = np.float64 if precision == "fp64" else np.int32
+    buf = torch.zeros(pic.pic_particles_raw_size(sim, n), dtype=torch.uint8).pin_memory()
+    raw, at = buf.numpy(), 0
+    for a, t in ((tri, np.int32), (l0, lam), (l1, lam), (u[:, 0], real), (u[:, 1], real), (u[:, 2], real)):
+        size = np.dtype(t).itemsize
+        raw[at:at + size * n] = np.ascontiguousarray(a, t).view(np.uint8)
+        at += size * stride
+    pic.pic_particles_raw_set(sim, buf.data_ptr(), n)
+    torch.cuda.synchronize()
+
+
+def _gradients(arrays):
+    """grad lambda_k (z, rho) of every triangle, in the mesh's counter-clockwise node order"""
+    p = np.asarray(arrays[0])[np.asarray(arrays[1])]
+    e = np.stack([p[:, (k + 2) % 3] - p[:, (k + 1) % 3] for k in range(3)], 1)
+    twice = (p[:, 1, 0] - p[:, 0, 0]) * (p[:, 2, 1] - p[:, 0, 1]) - \
+            (p[:, 2, 0] - p[:, 0, 0]) * (p[:, 1, 1] - p[:, 0, 1])
+    return np.stack([-e[:, :, 1], e[:, :, 0]], 2) / twice[:, None, None], twice
+
+
+@pytest.mark.parametrize("share", [0.0, 0.3, 0.7, 0.95])
+@pytest.mark.parametrize("below", [1.1e-16, 1e-12])
+def test_coordinate_below_zero_moving_inward(pic, below, share):
+    """FP64: on every edge (walls and the axis among them), `below` outside of its triangle,
+    at rest or moving inward by a share of that: the particle stays where it is."""
+    arrays = W.cavity_mesh(n_tri=400)
+    g, twice = _gradients(arrays)
+    N2 = len(twice)
+    assert np.all(twice > 0)   # the mesh keeps the node order of counter-clockwise triangles
+    arrays, sim, dt = _sim(pic, "fp64", 3 * N2)
+    tri = np.repeat(np.arange(N2), 3)
+    k = np.tile(np.arange(3), N2)
+    l = np.full((3 * N2, 3), 0.5)
+    l[np.arange(3 * N2), k] = -below
+    l[k == 2, 1] = 0.5 + max(below, 2.0 ** -53)   # l2 = 1 - l0 - l1
+    gk = g[tri, k]
+    v = share * below * gk / (gk ** 2).sum(1)[:, None] / dt
+    u = np.stack([v[:, 1], np.zeros(3 * N2), v[:, 0]], 1)
+    # one particle of each id through the ordinary way first: a species has to be known
+    centre = np.asarray(arrays[0])[np.asarray(arrays[1])].mean(1)[tri]
+    zero = np.zeros(3 * N2)
+    pic.pic_particles_inject(sim, centre[:, 0], centre[:, 1], zero, zero, zero, -1.0, 1.0, 1e-15)
+    ids = pic.pic_particles_get(sim)["pid"]
+    _raw_state(pic, sim, "fp64", tri, l[:, 0], l[:, 1], u)
+    pic.pic_step(sim, 1)
+    got, lam, gu = _by_pid(pic.pic_particles_get(sim), 3 * N2)
+    order = np.empty(3 * N2, np.int64)
+    order[ids] = np.arange(3 * N2)   # slot of each id
+    assert np.all(got >= 0) and np.all(np.isfinite(lam)) and np.all(np.isfinite(gu))
+    was = _positions(arrays, tri, np.stack([l[:, 0], l[:, 1], 1 - l[:, 0] - l[:, 1]], 1))[order]
+    assert np.abs(_positions(arrays, got, lam) - was).max() < 4 * below + 1e-14
+    d = pic.pic_diagnostics(sim, fields=True)
+    assert d["n_absorbed"] == 0 and np.all(np.isfinite(d["J"])) and np.all(np.isfinite(d["E"]))
