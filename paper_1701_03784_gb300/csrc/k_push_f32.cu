@@ -69,9 +69,9 @@ __device__ __forceinline__ int f2fix(float x) {
 }
 
 // Reciprocal and reciprocal square root of numbers in the normal range: the hardware's
-// approximations alone.  (__fdividef and rsqrtf wrap them in scaling for denormals, whose
-// instructions this kernel, bound by its issue rate, would pay in every push and segment;
-// in the normal range the values are the same.)
+// approximations alone, to which smaller ones are zero.  (__fdividef and rsqrtf wrap them in
+// scaling for denormals, whose instructions this kernel, bound by its issue rate, would pay
+// in every push and segment; in the normal range the values are the same.)
 __device__ __forceinline__ float rcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -82,6 +82,10 @@ __device__ __forceinline__ float rsq(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+
+// Fraction of a step from coordinate f (0 or 2^-22 at least) to le < 0 at which it is zero.
+// From f = 0 the step itself may be below the normal range: held there, the product is 0.
+__device__ __forceinline__ float zero_at(float f, float le) { return f * rcp(fmaxf(f - le, FLT_MIN)); }
 
 __device__ __forceinline__ const float4 *rec4(const TriRec<float> *rec, int t) {
     return reinterpret_cast<const float4 *>(rec + t);
@@ -152,9 +156,9 @@ __device__ __forceinline__ Seg segment_end(float f0, float f1, float f2, float d
         }
         return r;
     }
-    const float sA = x0 ? f0 * rcp(f0 - le0) : 2.f;
-    const float sB = x1 ? f1 * rcp(f1 - le1) : 2.f;
-    const float sC = x2 ? f2 * rcp(f2 - le2) : 2.f;
+    const float sA = x0 ? zero_at(f0, le0) : 2.f;
+    const float sB = x1 ? zero_at(f1, le1) : 2.f;
+    const float sC = x2 ? zero_at(f2, le2) : 2.f;
     if (sA <= sB && sA <= sC) { r.kx = 0; r.sx = sA; }
     else if (sB <= sC) { r.kx = 1; r.sx = sB; }
     else { r.kx = 2; r.sx = sC; }
@@ -462,7 +466,7 @@ __device__ __forceinline__ unsigned walk_pass(const PushArgs<PF32> &a, const QEn
         const float leP = fP + dP, leQ = fQ + dQ;
         const bool xP = leP < 0.f, xQ = leQ < 0.f, leaves = xP || xQ;
         // leaving: the edge reached first, opposite P or opposite Q, and the point on it
-        float sP = fP * rcp(fP - leP), sQ = fQ * rcp(fQ - leQ);
+        float sP = zero_at(fP, leP), sQ = zero_at(fQ, leQ);
         sP = xP ? sP : 2.f;
         sQ = xQ ? sQ : 2.f;
         const bool atP = j == 1 ? sP < sQ : sP <= sQ;   // the lower edge where both are reached at once

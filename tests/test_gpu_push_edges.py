@@ -1,6 +1,6 @@
-"""Particles at places that the particle kernels meet rarely: landing exactly on the axis, and
-coordinates that rounding left just below zero.  Force-free, so every particle ends at
-z + v_z dt, |rho + v_rho dt|."""
+"""Particles at places that the particle kernels meet rarely: landing exactly on the axis,
+coordinates that rounding left just below zero, and steps too small for a normal FP32 number.
+Force-free, so every particle ends at z + v_z dt, |rho + v_rho dt|."""
 import numpy as np
 import pytest
 
@@ -143,3 +143,41 @@ def test_coordinate_below_zero_moving_inward(pic, below, share):
     assert np.abs(_positions(arrays, got, lam) - was).max() < 4 * below + 1e-14
     d = pic.pic_diagnostics(sim, fields=True)
     assert d["n_absorbed"] == 0 and np.all(np.isfinite(d["J"])) and np.all(np.isfinite(d["E"]))
+
+
+@pytest.mark.parametrize("place", ["edge", "node"])
+@pytest.mark.parametrize("step", [1e-37, 1e-38, 1e-41])
+def test_step_below_the_normal_range(pic, step, place):
+    """FP32: at coordinate 0 of a triangle away from the walls, moving outward by a step of
+    `step` of that coordinate, a normal or a subnormal number: the particle stays where it is."""
+    arrays = W.cavity_mesh(n_tri=400)
+    g, _ = _gradients(arrays)
+    nodes, tris = np.asarray(arrays[0]), np.asarray(arrays[1])
+    wall = np.zeros(len(nodes), bool)
+    wall[np.asarray(arrays[2]).ravel()] = True
+    inner = np.flatnonzero(~wall[tris].any(1))
+    n = 3 * len(inner)
+    arrays, sim, dt = _sim(pic, "fp32", n)
+    tri, k = np.repeat(inner, 3), np.tile(np.arange(3), len(inner))
+    one, i = 1 << 22, np.arange(n)
+    l = np.full((n, 3), one // 2)
+    l[i, k] = 0
+    if place == "node":   # node k+1, leaving through edge k
+        l[i, (k + 1) % 3] = one
+        l[i, (k + 2) % 3] = 0
+    gk = g[tri, k]
+    v = -step * gk / (gk ** 2).sum(1)[:, None] / dt
+    u = np.stack([v[:, 1], np.zeros(n), v[:, 0]], 1)
+    centre = nodes[tris].mean(1)[tri]
+    zero = np.zeros(n)
+    pic.pic_particles_inject(sim, centre[:, 0], centre[:, 1], zero, zero, zero, -1.0, 1.0, 1e-15)
+    ids = pic.pic_particles_get(sim)["pid"]
+    _raw_state(pic, sim, "fp32", tri, l[:, 0], l[:, 1], u)
+    pic.pic_step(sim, 1)
+    got, lam, _ = _by_pid(pic.pic_particles_get(sim), n)
+    order = np.empty(n, np.int64)
+    order[ids] = i
+    assert np.all(got >= 0)
+    was = _positions(arrays, tri, l / one)[order]
+    assert np.abs(_positions(arrays, got, lam) - was).max() < 1e-6
+    assert pic.pic_diagnostics(sim)["n_absorbed"] == 0
