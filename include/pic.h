@@ -457,8 +457,12 @@ pic_status pic_launch_count(int64_t *out);
  * the training batch and the rows of pic_mlp_grad; inference is chunked.  Limits:
  * 1..64 members, 1..16 layers, widths 1..4096, max_batch 1..2^20.  Host arrays are
  * caller-owned and copied; device arrays (X, T, Y) are caller-owned CUDA memory on the
- * network's device.  Errors of every call: ARG (null handle or pointer, a limit above),
- * OOM, CUDA, and TIMEOUT where stated; pic_mlp_destroy releases everything. */
+ * network's device.  Calls on one network share its scratch memory, so the caller orders
+ * those on different streams (an event, a synchronisation); only FP32 forward calls on more
+ * than min(2 max_batch, 1024) rows with every width at most 256 use none and may overlap each
+ * other.  A recorded FP32 forward call reads the parameters of the time of its replay.
+ * Errors of every call: ARG (null handle or pointer, a limit above), OOM, CUDA, and TIMEOUT
+ * where stated; pic_mlp_destroy releases everything. */
 typedef struct pic_mlp pic_mlp;
 pic_status pic_mlp_create(int32_t n_members, int32_t n_layers, const int32_t *sizes,
                           int32_t max_batch, pic_mlp **out);
