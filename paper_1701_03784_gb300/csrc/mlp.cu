@@ -87,13 +87,15 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long x) {
 
 // `rows` samples per member into the member's batch buffers (row stride mrows): drawn from
 // n with replacement (random = 1) or rows 0.. of X and T (random = 0).  One thread a value:
-// one thread a row, looping over its 6 + 33 values, took 8.4 us for 5 x 128 rows.
+// one thread a row, looping over its 6 + 33 values, took 8.4 us for 5 x 128 rows.  Clears the
+// members' losses for the kernels behind it, where they are wanted.
 __global__ void k_gather(const float *X, const float *T, float *Xb, float *Tb, long long n, int rows,
                          int mrows, int din, int dout, unsigned long long seed, long long step,
-                         int random) {
+                         int random, float *loss) {
     chain_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int z = blockIdx.y, w = din + dout;
+    if (loss && i == 0) loss[z] = 0.f;
     const int r = (int)(i / w), k = (int)(i % w);
     if (r >= rows) return;
     long long s = r;
@@ -465,9 +467,9 @@ struct MlpImpl {
     }
 
     void gather(int rows, const float *X, const float *T, long long n, unsigned long long seed,
-                long long step, int random, bool chain, cudaStream_t s) {
+                long long step, int random, float *loss_out, bool chain, cudaStream_t s) {
         launch_chained(chain, k_gather, dim3(blocks((long long)rows * (sz[0] + sz[L])), E), 256, 0, s, X, T, act[0],
-                       Tb, n, rows, max_batch, sz[0], sz[L], seed, step, random);
+                       Tb, n, rows, max_batch, sz[0], sz[L], seed, step, random, loss_out);
     }
     // FP32 inference on n rows by the whole-network kernel, or layer by layer in batches of
     // max_batch.  A block of the whole-network kernel takes as long for one row as for its
@@ -651,8 +653,7 @@ extern "C" pic_status pic_mlp_grad(pic_mlp *m, const float *X, const float *T, i
     }
     cudaStream_t s = (cudaStream_t)st;
     const int rows = (int)n;
-    x.gather(rows, X, T, n, 0, 0, 0, false, s);
-    PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
+    x.gather(rows, X, T, n, 0, 0, 0, x.loss, false, s);
     if (x.train_tc) {
         x.forward(rows, x.act[0], (long long)x.max_batch * x.sz[0], s);
         x.backward(rows, x.loss, s);
@@ -684,9 +685,8 @@ extern "C" pic_status pic_mlp_train(pic_mlp *m, const float *X, const float *T, 
     const long long np = x.E * x.P;
     x.tc_dirty = true;
     for (long long k = 0; k < steps; k++) {
-        x.gather(batch, X, T, n, seed, x.adam_step, 1, k > 0, s);
         const bool last = k == steps - 1;
-        if (last) PIC_CUDA_TRY(cudaMemsetAsync(x.loss, 0, sizeof(float) * x.E, s));
+        x.gather(batch, X, T, n, seed, x.adam_step, 1, last ? x.loss : nullptr, k > 0, s);
         x.adam_step++;
         const float b1 = 0.9f, b2 = 0.999f;
         const AdamArgs adam{(float)lr, b1, b2, 1e-8f, 1.f - std::pow(b1, (float)x.adam_step),
