@@ -21,12 +21,16 @@ namespace pic {
 
 namespace {
 
-// Block g of a recorder's n groups: term(k) summed over the group's entries when due
+// Block g of a recorder's n groups: term(k) summed over the group's entries when due.  The
+// sum is that of PARTS strided parts, folded the same way whatever the block's size (a
+// multiple of 32): what is recorded does not depend on the launch shape that a tuner picks.
+constexpr int PARTS = 256;
+
 template <class Term>
 __device__ __forceinline__ void record_block(int g, int n, const int64_t *ptr, long long *state,
                                              unsigned *done, int every, long long capacity, double *buf,
                                              Term term) {
-    __shared__ double part[16];
+    __shared__ double part[PARTS / 32];
     __shared__ long long s_step, s_rec;
     if (threadIdx.x == 0) {
         s_step = state[0];
@@ -35,10 +39,12 @@ __device__ __forceinline__ void record_block(int g, int n, const int64_t *ptr, l
     __syncthreads();
     const bool take = s_step % every == 0;
     if (take) {
-        double s = 0.0;
-        for (long long k = ptr[g] + threadIdx.x; k < ptr[g + 1]; k += blockDim.x) s += term(k);
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+        for (int v = threadIdx.x; v < PARTS; v += blockDim.x) {   // whole warps
+            double s = 0.0;
+            for (long long k = ptr[g] + v; k < ptr[g + 1]; k += PARTS) s += term(k);
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((v & 31) == 0) part[v >> 5] = s;
+        }
         __syncthreads();
     }
     // every block has read the counters before it takes its ticket; the last one advances
@@ -46,7 +52,7 @@ __device__ __forceinline__ void record_block(int g, int n, const int64_t *ptr, l
     if (threadIdx.x == 0) {
         if (take && s_rec < capacity) {
             double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += part[w];
+            for (int w = 0; w < PARTS / 32; w++) t += part[w];
             buf[s_rec * n + g] = t;
         }
         __threadfence();
