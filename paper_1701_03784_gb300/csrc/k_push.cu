@@ -45,7 +45,8 @@ __device__ __forceinline__ int sel3(int k, int a, int b, int c) { return k == 0 
 
 constexpr int PW = 2;        // warps per block: few particles spread over all SMs' FP64 units
 constexpr int QCAP = 64;     // ring entries per warp (at most 31 + 32 used)
-constexpr int ROUNDS = 8;    // slots a warp takes at most: 32 ROUNDS
+constexpr int ROUNDS = 8;    // 32 ROUNDS slots a warp are enough to fill its ring
+constexpr int BPS = 16;      // blocks resident per SM (at most 64 registers a thread)
 
 // particles whose displacement (d0, d1) leaves triangle t, at l = (l0, l1, 1 - l0 - l1)
 struct Ring {
@@ -216,7 +217,7 @@ __device__ __forceinline__ unsigned walk(const PushArgs<PF64> &a, int slot, int 
 }  // namespace
 
 template <bool VAY>
-__global__ void __launch_bounds__(32 * PW) k_push_f64(const __grid_constant__ PushArgs<PF64> a) {
+__global__ void __launch_bounds__(32 * PW, BPS) k_push_f64(const __grid_constant__ PushArgs<PF64> a) {
     __shared__ Ring rings[PW];
     chain_wait();
     const int64_t n = *a.n_slots;
@@ -231,9 +232,7 @@ __global__ void __launch_bounds__(32 * PW) k_push_f64(const __grid_constant__ Pu
         __syncwarp();
     };
     // the rounds of 32 slots in use are dealt out evenly: of the slots that the launch allows
-    // for there may be few (with an emitter, it allows for the capacity).  50,000 in room for
-    // 3M, each warp its eight rounds until there are no more: 53 us; dealt out: 36 us; in room
-    // for 51,000: 31 us
+    // for there may be few (with an emitter, it allows for the capacity)
     const unsigned long long all = (unsigned long long)(n + 31) / 32, warps = (unsigned long long)gridDim.x * PW;
     const unsigned me = blockIdx.x * PW + warp;
     const int64_t last = (int64_t)(32 * ((me + 1) * all / warps));
@@ -315,12 +314,16 @@ static void launch_push_f64(const PushArgs<PF64> &a, int64_t n_bound, cudaStream
     cudaGetDevice(&dev);
     int &sm = sms[dev & 63];
     if (sm == 0) cudaDeviceGetAttribute(&sm, cudaDevAttrMultiProcessorCount, dev);
-    // as many slots a warp as keep 16 warps on every SM, up to ROUNDS of 32: more of them
-    // fill the last ring pass better, fewer spread a small simulation over the SMs
-    const int64_t all = (n_bound + 31) / 32;
-    const int rounds = (int)std::min<int64_t>(ROUNDS, std::max<int64_t>(1, all / (16 * std::max(sm, 1))));
-    const int64_t warps = (all + rounds - 1) / rounds;
-    const unsigned grid = (unsigned)((warps + PW - 1) / PW);
+    // As many slots a warp as keep 16 warps on every SM, up to ROUNDS of 32: more of them
+    // fill the last ring pass better, fewer spread a small simulation over the SMs; and no
+    // more blocks than fit at a time.  Room for 3M, us a launch with 1000, 50,000, 1M slots in
+    // use: ROUNDS in a row for each warp 47, 50, 266; dealt out over as many warps as ROUNDS for
+    // 3M ask 18, 34, 286; over those that fit 17, 31, 262.  All slots in use, launches of 1.25M,
+    // 4M, 12M: 307, 896, 2637 -> 291, 883, 2585
+    const int64_t all = (n_bound + 31) / 32, spread = 16 * std::max(sm, 1);
+    const int64_t rounds = std::min<int64_t>(ROUNDS, std::max<int64_t>(1, all / spread));
+    const int64_t blocks = ((all + rounds - 1) / rounds + PW - 1) / PW;
+    const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)BPS * std::max(sm, 1));
     if (a.pusher == PIC_PUSHER_VAY) launch_chained(a.chain, k_push_f64<true>, grid, 32 * PW, 0, s, a);
     else launch_chained(a.chain, k_push_f64<false>, grid, 32 * PW, 0, s, a);
 }
