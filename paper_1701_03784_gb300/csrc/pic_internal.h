@@ -227,7 +227,9 @@ inline void edge_tail_head(const int32_t *n3, int k, int *a, int *b) {
 }
 
 // run f(begin, end) over [0, n) on the host's cores, at least `grain` items a thread: a
-// thread takes some 30 us to start, so light loops ask for thousands
+// thread takes some 30 us to start, so light loops ask for thousands.  The caller takes a part
+// too, and the parts of threads that do not start.  An exception thrown by f is thrown on
+// once every thread is done (the first part's of several).
 template <class F>
 void parallel_for(int64_t n, F &&f, int64_t grain = 1) {
     unsigned nt = std::max(1u, std::min(64u, std::thread::hardware_concurrency()));
@@ -236,14 +238,29 @@ void parallel_for(int64_t n, F &&f, int64_t grain = 1) {
         f((int64_t)0, n);
         return;
     }
+    const int64_t chunk = (n + nt - 1) / nt;
+    std::vector<std::exception_ptr> thrown(nt);
+    const auto part = [&](unsigned i) {
+        const int64_t a = std::min(n, (int64_t)i * chunk), b = std::min(n, a + chunk);
+        if (a >= b) return;
+        try {
+            f(a, b);
+        } catch (...) {
+            thrown[i] = std::current_exception();
+        }
+    };
     std::vector<std::thread> th;
-    int64_t chunk = (n + nt - 1) / nt;
-    for (unsigned i = 0; i < nt; i++) {
-        int64_t a = (int64_t)i * chunk, b = std::min(n, a + chunk);
-        if (a >= b) break;
-        th.emplace_back([=, &f] { f(a, b); });
+    th.reserve(nt);   // nothing below throws but the start of a thread
+    unsigned started = 1;
+    try {
+        for (; started < nt; started++) th.emplace_back(part, started);
+    } catch (...) {
     }
+    part(0);
+    for (unsigned i = started; i < nt; i++) part(i);
     for (auto &t : th) t.join();
+    for (const auto &e : thrown)
+        if (e) std::rethrow_exception(e);
 }
 
 void build_locator(HostMesh &m);
