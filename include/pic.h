@@ -124,8 +124,9 @@ pic_status pic_set_allocator(pic_alloc_fn alloc, pic_free_fn free_, void *ctx);
  * (Eq. dis_hodge_mu: rho_bar_f / (mu0 A_f)).  Host-only; no device memory yet.
  * The mesh must be conforming: an edge belongs to one or two triangles, and two triangles
  * sharing an edge lie on opposite sides of it (either node order is accepted per triangle).
- * Errors: PIC_ERR_ARG (null / non-positive sizes / rho < 0 / bad index), PIC_ERR_MESH
- * (degenerate or overlapping triangles, an edge in three triangles, bad boundary list). */
+ * Errors: PIC_ERR_ARG (null / non-positive sizes / 2^29 triangles or more / rho < 0 / bad
+ * index), PIC_ERR_MESH (degenerate or overlapping triangles, an edge in three triangles, bad
+ * boundary list). */
 pic_status pic_mesh_create(const double *nodes_zr, int64_t n_nodes, const int32_t *tris,
                            int64_t n_tris, const int32_t *bedge_nodes,
                            const int32_t *bedge_tag, int64_t n_bedges, const pic_units *u,

@@ -168,7 +168,8 @@ extern "C" pic_status pic_mesh_create(const double *nodes_zr, int64_t n_nodes,
         set_error("pic_mesh_create: null pointer or bad size");
         return PIC_ERR_ARG;
     }
-    if (n_nodes >= (int64_t)1 << 31 || n_tris >= (int64_t)1 << 30) {
+    // 4 x triangle + a part of it (edge_face, node_face, the re-sort's keys) has 31 bits
+    if (n_nodes >= (int64_t)1 << 31 || n_tris >= (int64_t)1 << 29) {
         set_error("pic_mesh_create: mesh too large for 32-bit indices");
         return PIC_ERR_ARG;
     }
