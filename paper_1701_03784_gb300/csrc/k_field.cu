@@ -90,9 +90,9 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
     if constexpr (LOSS) Bnew = a.loss_f[2 * f] * Bold - a.loss_f[2 * f + 1] * (a.dt * curl);
     a.B[f] = Bnew;
     if constexpr (P::fixed) {
-        longlong2 *fs = reinterpret_cast<longlong2 *>(a.face + f);
-        fs[0] = make_longlong2(0, 0);
-        fs[1] = make_longlong2(0, __double_as_longlong((double)mu * (double)Bnew));
+        FaceSum &fs = a.face[f];
+        *reinterpret_cast<longlong2 *>(&fs.d0) = make_longlong2(0, 0);
+        *reinterpret_cast<longlong2 *>(&fs.a1) = make_longlong2(0, __double_as_longlong((double)mu * (double)Bnew));
     }
     R w[8];
 #pragma unroll
@@ -181,8 +181,9 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
             if (fs[q] == 0) continue;
             const int fk = abs(fs[q]) - 1, f = fk >> 2;
             if constexpr (P::fixed) {
-                const longlong2 *F = reinterpret_cast<const longlong2 *>(a.face + f);
-                const longlong2 d = F[0], ah = F[1];
+                const FaceSum &sum = a.face[f];
+                const longlong2 d = *reinterpret_cast<const longlong2 *>(&sum.d0);
+                const longlong2 ah = *reinterpret_cast<const longlong2 *>(&sum.a1);
                 long long A = ah.x;                                  // edge 1
                 if ((fk & 3) != 1) A += d.x << LAM_BITS;             // edge 2
                 if ((fk & 3) == 0) A += d.y << LAM_BITS;             // edge 0
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(512) k_field_r(const __grid_constant__ FieldAr
     if constexpr (P::fixed) {
         long long out = 0;
         const auto left = [&](int fk) {
-            const longlong2 d = *reinterpret_cast<const longlong2 *>(a.face + (fk >> 2));
+            const longlong2 d = *reinterpret_cast<const longlong2 *>(&a.face[fk >> 2].d0);
             const int k = fk & 3;
             out += k == 0 ? d.x : k == 1 ? d.y : -(d.x + d.y);
         };

@@ -175,10 +175,10 @@ __device__ __forceinline__ Seg segment_end(float f0, float f1, float f2, float d
 // adds a triangle's current sums of this warp, or of one segment (FaceSum)
 __device__ __forceinline__ void add_current(const PushArgs<PF32> &a, int t, long long a1, long long d0,
                                             long long d1) {
-    unsigned long long *f = reinterpret_cast<unsigned long long *>(a.face + t);
-    atomicAdd(f, (unsigned long long)d0);
-    atomicAdd(f + 1, (unsigned long long)d1);
-    atomicAdd(f + 2, (unsigned long long)a1);
+    FaceSum &f = a.face[t];
+    atomicAdd(&f.d0, (unsigned long long)d0);
+    atomicAdd(&f.d1, (unsigned long long)d1);
+    atomicAdd(&f.a1, (unsigned long long)a1);
 }
 
 // a particle whose displacement leaves its start triangle t: slot, start point (s0, s1,

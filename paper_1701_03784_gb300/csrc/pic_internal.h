@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdint>
 #include <exception>
 #include <new>
@@ -356,10 +357,16 @@ struct alignas(sizeof(R) == 4 ? 128 : 64) TriRec {
 //   A2 - A1 = 2^22 (s0 - e0),  A0 - A2 = 2^22 (s1 - e1)   (the identity behind Eq. DCE),
 // so one product pair (A1) and two differences determine all three, also after summing
 // over the segments in the triangle; and the charge that leaves node k through the
-// triangle is the sum of s_k - e_k.
+// triangle is the sum of s_k - e_k.  Beside the sums, in the same 32-byte sector, what the
+// residual kernel needs of the triangle's B.  Read and written in 16-byte words.
 struct alignas(32) FaceSum {
-    long long a1, d0, d1, pad;
+    unsigned long long d0, d1;   // sums of s0 - e0 and s1 - e1 (two's complement)
+    unsigned long long a1;       // sum of A1
+    double h;                    // star_mu^-1 B^{n+1/2}
 };
+static_assert(offsetof(FaceSum, d0) == 0 && offsetof(FaceSum, d1) == 8 && offsetof(FaceSum, a1) == 16 &&
+                  offsetof(FaceSum, h) == 24 && sizeof(FaceSum) == 32,
+              "d0, d1 and a1, h are a 16-byte word each");
 
 struct PF32 {
     using R = float;
