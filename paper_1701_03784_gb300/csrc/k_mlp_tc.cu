@@ -689,7 +689,10 @@ bool mlp_tc_gemm(const TcGemmOp &g, int E, uint16_t *scratch_a, uint16_t *scratc
 // How many pairs of SMs share a member's `tiles`, of `slots` pairs that fit at a time: the
 // count with the shortest time, taken as the rounds of pairs times a pair's time, in units of
 // two tiles' pass through the layers.  A single tile's pass takes about 3/4 (nothing overlaps
-// its epilogues), starting and leaving about 1/4.
+// its epilogues), starting and leaving about 1/4.  Against the best of some 30 counts (us a
+// call, this rule / best): 5 members of 4 x 256 at 4000, 20000, 65536, 131072 rows 51 / 49, 89 / 88,
+// 199 / 199, 365 / 365; 8 of 2 x 100 at the same 39 / 39, 67 / 67, 135 / 135, 241 / 241; one of 4 x 256
+// 48 / 46, 51 / 49, 71 / 68, 105 / 104; 5 of 4 x 64 40 / 38, 58 / 58, 112 / 112, 195 / 193.
 static unsigned pairs_per_member(long long tiles, int E, int slots) {
     long long best = 1;
     double least = 0;

@@ -186,9 +186,14 @@ struct SimImpl final : SimBase {
 
     bool timing_on = false;
     // host round trips (step_host): uploads and downloads run on streams of their own,
-    // chunk by chunk (8M slots, ms for four steps: 3, 4, 6 chunks -> 5.56, 5.53, 5.55; fewer
-    // leave a longer pipeline to fill and drain, more pay for launches and copies)
+    // chunk by chunk.  More chunks leave a shorter pipeline to fill and drain, once a call, and
+    // cost a launch and two copies each, every step (10 to 16 us): RT_CHUNKS where the
+    // state is large for the number of steps, one less otherwise.  us a step with 2, 3, 4, 6
+    // chunks, calls of 4 steps and of 32: 1M slots 205, 190, 197, 195 and 187, 174, 184, 202;
+    // 8M 1317, 1239, 1230, 1234 and 1237, 1176, 1184, 1202; 16M 2585, 2431, 2404, 2390 and 2435,
+    // 2317, 2328, 2347
     static constexpr int RT_CHUNKS = 4;
+    static int round_trip_chunks(int64_t n, int64_t steps) { return n >> 20 > steps ? RT_CHUNKS : RT_CHUNKS - 1; }
     // CUDA-graph replay of whole periods of steps (2 x the re-sort interval: the buffer
     // parities and the re-sort phase are back where they started)
     bool use_graph = false, stepped = false;
@@ -1439,16 +1444,17 @@ struct SimImpl final : SimBase {
     // copies: chunk c is uploaded once the previous step's write-back of it is done,
     // pushed once it has landed, and written back once it is pushed (or, on a re-sort
     // step, once the re-sort is done)
-    pic_status step_host_pipelined(char *h, int64_t n, int64_t chunk, bool first, cudaStream_t s) {
+    pic_status step_host_pipelined(char *h, int64_t n, int64_t chunk, int chunks, bool first,
+                                   cudaStream_t s) {
         pic_status st;
         stepped = true;
         FieldArgs<P> fa = field_args();
         fa.chain = false;
         if ((st = step_begin(fa, s)) != PIC_OK) return st;
-        k_chunk_counts<<<1, 32, 0, s>>>(d_n, d_chunk_n, chunk, RT_CHUNKS);
+        k_chunk_counts<<<1, 32, 0, s>>>(d_n, d_chunk_n, chunk, chunks);
         PIC_LAUNCHED();
         const bool resort_due = sort_interval > 0 && since_sort + 1 >= sort_interval;
-        for (int c = 0; c < RT_CHUNKS; c++) {
+        for (int c = 0; c < chunks; c++) {
             const int64_t c0 = std::min(n, c * chunk), c1 = std::min(n, c0 + chunk);
             if (!first) PIC_CUDA_TRY(cudaStreamWaitEvent(up_stream, rt_chunk[c], 0));
             if (c1 > c0 && (st = copy_slots(h, n, c0, c1, true, up_stream)) != PIC_OK) return st;
@@ -1480,7 +1486,7 @@ struct SimImpl final : SimBase {
         if (resort_due) {
             PIC_CUDA_TRY(cudaEventRecord(rt_step, s));
             PIC_CUDA_TRY(cudaStreamWaitEvent(rt_stream, rt_step, 0));
-            for (int c = 0; c < RT_CHUNKS; c++) {
+            for (int c = 0; c < chunks; c++) {
                 const int64_t c0 = std::min(n, c * chunk), c1 = std::min(n, c0 + chunk);
                 if (c1 > c0 && (st = copy_slots(h, n, c0, c1, false, rt_stream)) != PIC_OK)
                     return st;
@@ -1513,7 +1519,8 @@ struct SimImpl final : SimBase {
         char *h = static_cast<char *>(state);
         // chunks of whole particle-kernel tiles (512 slots), so that a chunk's tiles read
         // none of the next chunk's slots
-        const int64_t chunk = ((n + RT_CHUNKS - 1) / RT_CHUNKS + 511) / 512 * 512;
+        const int chunks = round_trip_chunks(n, steps);
+        const int64_t chunk = ((n + chunks - 1) / chunks + 511) / 512 * 512;
         // FP32 build (without kernel timing): each chunk is pushed as soon as it has landed and
         // written back as soon as it is pushed, so the step's particle work overlaps both
         // copy directions; the E update and any re-sort follow the last chunk (a re-sort
@@ -1534,12 +1541,12 @@ struct SimImpl final : SimBase {
                     n_bound = n;
                     dgl_dirty = true;
                 }
-                if ((st = step_host_pipelined(h, n, chunk, k == 0, s)) != PIC_OK) return st;
+                if ((st = step_host_pipelined(h, n, chunk, chunks, k == 0, s)) != PIC_OK) return st;
                 continue;
             }
             // upload; chunk c waits only for the previous step's download of chunk c, so the
             // two copy directions overlap
-            for (int c = 0; c < RT_CHUNKS; c++) {
+            for (int c = 0; c < chunks; c++) {
                 const int64_t c0 = std::min(n, c * chunk), c1 = std::min(n, c0 + chunk);
                 if (k > 0) PIC_CUDA_TRY(cudaStreamWaitEvent(up_stream, rt_chunk[c], 0));
                 if (c1 > c0 && (st = copy_slots(h, n, c0, c1, true, up_stream)) != PIC_OK)
@@ -1556,7 +1563,7 @@ struct SimImpl final : SimBase {
             if ((st = step(1, s)) != PIC_OK) return st;
             PIC_CUDA_TRY(cudaEventRecord(rt_step, s));
             PIC_CUDA_TRY(cudaStreamWaitEvent(rt_stream, rt_step, 0));
-            for (int c = 0; c < RT_CHUNKS; c++) {
+            for (int c = 0; c < chunks; c++) {
                 const int64_t c0 = std::min(n, c * chunk), c1 = std::min(n, c0 + chunk);
                 if (c1 > c0 && (st = copy_slots(h, n, c0, c1, false, rt_stream)) != PIC_OK)
                     return st;
