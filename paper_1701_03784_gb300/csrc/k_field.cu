@@ -110,7 +110,9 @@ __global__ void __launch_bounds__(512) k_field_b(const __grid_constant__ FieldAr
 }
 
 // A 64-bit integer as a double in two FP64 additions: each half becomes the low bits of a
-// double's mantissa (at 2^52 and 2^84), whose offsets are then taken out.
+// double's mantissa (at 2^52 and 2^84), whose offsets are then taken out.  The first addition
+// is exact (multiples of 2^32 that come out below 2^64), the second rounds once: the nearest
+// double.
 __device__ __forceinline__ double to_double(long long v) {
     const double lo = __hiloint2double(0x43300000, (int)v);                                   // 2^52 + low
     const double hi = __hiloint2double(0x45300000, (int)((unsigned)(v >> 32) ^ 0x80000000u)); // 2^84 + (high + 2^31) 2^32

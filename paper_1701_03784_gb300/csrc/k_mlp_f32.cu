@@ -351,7 +351,9 @@ int sm_count() {
 // activations and 8 weights and issues 4 TR packed FMAs (fma.rn.f32x2: two rows an
 // instruction, which leaves issue slots for the shared-memory reads).  TR follows the
 // layer's width, so that a narrow output layer is spread over all threads too.  Each
-// element's sum runs over k in order, the same chain as in the layer products.
+// element's sum runs over k in order, as in the 64 x 64 tiles of the layer products; the
+// 32 x 32 tiles add eight partial sums, so that a row's last bits depend on the path that the
+// number of rows takes.
 constexpr int FNT = 256;      // threads
 constexpr int FK = 16;        // k a stage
 constexpr int FSTG = 3;
